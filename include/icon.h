@@ -456,16 +456,15 @@ void icon_domain_free(icon_domain* domain);
 
 /* Tile of a kernel kind (the kind numbers of icon_kernel_kind_name) of a mixed-precision
  * state. Stencil kinds (10, 11, 12, 13, 15, 16): lanes per entity (32 = one entity per
- * warp, 16 = two, 8 = four) and threads per block (64, 128, 256 or 512). The lean column
- * (24): its launch shape, lanes = the unroll factor of its two sweeps and block = the
- * resident 128-thread blocks per SM its registers are held to, one of (2, 9), (2, 10),
- * (2, 8), (2, 12), (2, 6); a tuned shape applies to the predictor's column, the
- * corrector's keeps (2, 9) unless a shape is forced. The autotuner picks them on the
- * first step (timing every candidate on the state's data, in the order of the step;
- * cached per grid size, level count and GPU,
- * and in the file named by the environment variable ICON_TUNE_CACHE if set). set_tiling
- * forces a tile (lanes 0 restores automatic choice; ICON_EINVAL for any other value
- * outside these sets); results do not depend on the tile. */
+ * warp, 16 = two, 8 = four) and threads per block (64, 128, 256 or 512); the autotuner
+ * picks them on the first step (timing every candidate on the state's data, in the order
+ * of the step; cached per grid size, level count and GPU, and in the file named by the
+ * environment variable ICON_TUNE_CACHE if set). The lean column (24): its launch form,
+ * lanes 2 and block one of 9 (chosen by the grid's size, the default), 6 or 8 (blocks of
+ * four or eight warps per 32 columns), 10 or 12 (one column per thread, its loads one or
+ * two levels ahead), the same in both stages. set_tiling forces a tile (lanes 0 restores
+ * automatic choice; ICON_EINVAL for any other value outside these sets); results do not
+ * depend on the tile. */
 int icon_state_tiling(const icon_state* state, int kind, int* lanes, int* block);
 int icon_state_set_tiling(icon_state* state, int kind, int lanes, int block);
 

@@ -1489,13 +1489,10 @@ __device__ inline void lean_flush(const MxGeo& G, const MxLeanArgs& a, const Lea
 }
 
 // one column per thread (lane); every lane of the warp runs the loops (lanes past the last
-// cell compute on zeros and store nothing) so that the chunk flushes stay warp-synchronous
-// TOPO (terrain-following levels): each cell's interpolation weights, 1/dz and 1/dzh and
-// reference Exner (level-major tables) in place of the per-level constants, the contravariant
-// (1 - beta) w - wcc in the explicit vertical fluxes (zero at the lid and the ground), the
-// gathered divergences scaled by the cell's 1/dz, and the stage's terrain-following w at the
-// ground
-template <bool CORR, int U, int CH, bool TOPO = false>
+// cell compute on zeros and store nothing) so that the chunk flushes stay warp-synchronous. The persistent
+// ensemble's form (a warp per 32 columns, every load in order, 64 registers); the per-state
+// kernels are in lean_column.h
+template <bool CORR, int U, int CH>
 __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, int64_t c, int64_t c0, int lane,
                                            LeanTile<CH>& T) {
   const int N = G.N, ld = G.ld;
@@ -1536,16 +1533,6 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
       ti = thv1;
       rif = rho1f;
       tif = thv1f;
-    } else if constexpr (TOPO) {
-      const double wu = LMV(a.t_wu_lm, j);
-      const float wuf = f64_to_f32(wu);
-      rif = wuf * rho1f + (1.0f - wuf) * rhof;
-      if (!CORR) {
-        ti = wu * thv1 + (1.0 - wu) * thv;
-        tif = f64_to_f32(ti);
-      } else {
-        tif = wuf * thv1f + (1.0f - wuf) * thvf;
-      }
     } else {
       rif = cf[LF_WU * ld + j] * rho1f + cf[LF_WL * ld + j] * rhof;
       if (!CORR) {
@@ -1558,39 +1545,21 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     const float Mh = rif * tif;
     const double wh = (j == 0 || j == N) ? 0.0 : LMV(a.w, j);
     const float whf = f64_to_f32(wh);
-    // the explicit vertical velocity through half level j: w on flat levels (the factor
-    // 1 - beta is in the level constant), (1 - beta) w - wcc on terrain-following ones
-    float xvj = whf;
-    if constexpr (TOPO) xvj = (j == 0 || j == N) ? 0.0f : (float)(1.0 - kBeta) * whf - a.t_wcc[cc * ld + j];
+    // the explicit vertical velocity through half level j (the factor 1 - beta is in the
+    // level constant)
+    const float xvj = whf;
     float gam1 = 0.f, dpe1 = 0.f;
     if (j >= 1) {
       const int k = j - 1;
-      float dtk = LMV(a.dt32, k), dt1, dtb;
-      if constexpr (TOPO) {
-        const double idz = LMV(a.t_idz_lm, k);
-        dtk *= f64_to_f32(idz);
-        dt1 = f64_to_f32(dtau * idz);
-        dtb = f64_to_f32(dtau * kBeta * idz);
-      } else {
-        dt1 = cf[LF_DT1 * ld + k];
-        dtb = cf[LF_DTB * ld + k];
-      }
+      const float dtk = LMV(a.dt32, k), dt1 = cf[LF_DT1 * ld + k], dtb = cf[LF_DTB * ld + k];
       const float dthe = -dtk - dt1 * (M1 * xv1 - Mh * xvj);
       const float g = kRcvF * __fdividef(f64_to_f32(ex1), rho1f * thv1f);
       gam1 = g * dtb;
       dpe1 = g * dthe;
       if (k >= 1) {
         const int h = k;
-        double cpdzh;                                    // cpd / dzh of half level h
-        float ca;
-        if constexpr (TOPO) {
-          const double idzh = LMV(a.t_idzh_lm, h);
-          cpdzh = kCpd * idzh;
-          ca = f64_to_f32(dtau * kBeta * kCpd * idzh);
-        } else {
-          cpdzh = cd[LD_CPDZH * ld + h];
-          ca = cf[LF_CA * ld + h];
-        }
+        const double cpdzh = cd[LD_CPDZH * ld + h];      // cpd / dzh of half level h
+        const float ca = cf[LF_CA * ld + h];
         const float aa = ca * ti1f;
         const float lo = -aa * gam2 * M2;
         const float di = 1.0f + aa * (gam2 + gam1) * M1;
@@ -1645,7 +1614,6 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     ri_next = f64_to_f32(rho_k);
     M_next = ri_next * f64_to_f32(thv_k);
   }
-  const int64_t o = cc * ld;
 #pragma unroll U
   for (int k = N - 1; k >= 0; --k) {
     // half level k: the level above
@@ -1662,17 +1630,12 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     if (k == 0) {
       ri_k = rho_kf;
       M_k = rho_kf * thv_kf;
-    } else if constexpr (TOPO) {
-      const float wuf = f64_to_f32(LMV(a.t_wu_lm, k));
-      ri_k = wuf * f64_to_f32(rho_u) + (1.0f - wuf) * rho_kf;
-      M_k = ri_k * (wuf * f64_to_f32(thv_u) + (1.0f - wuf) * thv_kf);
     } else {
       ri_k = cf[LF_WU * ld + k] * f64_to_f32(rho_u) + cf[LF_WL * ld + k] * rho_kf;
       M_k = ri_k * (cf[LF_WU * ld + k] * f64_to_f32(thv_u) + cf[LF_WL * ld + k] * thv_kf);
     }
     const float wf_k = k >= 1 ? f64_to_f32(LMV(a.w, k)) : 0.0f;
-    float xv_k = wf_k;
-    if constexpr (TOPO) xv_k = k >= 1 ? (float)(1.0 - kBeta) * wf_k - a.t_wcc[o + k] : 0.0f;
+    const float xv_k = wf_k;
     // back substitution at half level k
     double x = 0.0, wn = 0.0;
     if (k >= 1) {
@@ -1681,19 +1644,8 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     }
     const float wnf = f64_to_f32(wn);
     // full level k
-    float dtb, dt1, dtk = LMV(a.dt32, k);
-    double idz = 0.0, exref;
-    if constexpr (TOPO) {
-      idz = LMV(a.t_idz_lm, k);
-      dtk *= f64_to_f32(idz);
-      dt1 = f64_to_f32(dtau * idz);
-      dtb = f64_to_f32(dtau * kBeta * idz);
-      exref = LMV(a.t_exref_lm, k);
-    } else {
-      dtb = cf[LF_DTB * ld + k];
-      dt1 = cf[LF_DT1 * ld + k];
-      exref = cd[LD_EXREF * ld + k];
-    }
+    const float dtk = LMV(a.dt32, k), dtb = cf[LF_DTB * ld + k], dt1 = cf[LF_DT1 * ld + k];
+    const double exref = cd[LD_EXREF * ld + k];
     const float dthe = -dtk - dt1 * (M_k * xv_k - M_next * xv_next);
     const float g = kRcvF * __fdividef(f64_to_f32(ex_k), rho_kf * thv_kf);
     const float q = M_k * wnf - M_next * wnf_next;
@@ -1701,25 +1653,16 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     const float dex = g * dthe - g * dtb * q;        // Exner increment (linearised state equation)
     float s_rho, s_thv, s_exp;
     if (!CORR) {
-      float drk = LMV(a.dr32, k);
-      if constexpr (TOPO) drk *= f64_to_f32(idz);
+      const float drk = LMV(a.dr32, k);
       const float drho = -drk - dt1 * (ri_k * xv_k - ri_next * xv_next) - dtb * (ri_k * wnf - ri_next * wnf_next);
       s_rho = rho_kf + drho;
       s_thv = thv_kf + __fdividef(dTh - drho * thv_kf, s_rho);
       s_exp = f64_to_f32(ex_k - exref) + dex;
       ok = ok && isfinite(s_thv) && isfinite(s_exp) && isfinite(wnf);
     } else {
-      // vertical mass flux through half level k of the step: rho_ic ((1 - beta) w^n + beta w^{n+1}),
-      // less rho_ic wcc on terrain-following levels
-      double t;
-      float fk;
-      if constexpr (TOPO) {
-        fk = ri_k * (xv_k + (float)kBeta * wnf);
-        t = fma(dtau * idz, f32_to_f64(fk) - f32_to_f64(fflux_next), LMV(a.dr64, k) * idz);
-      } else {
-        fk = ri_k * ((float)(1.0 - kBeta) * wf_k + (float)kBeta * wnf);
-        t = fma(cd[LD_IDZ * ld + k], f32_to_f64(fk) - f32_to_f64(fflux_next), LMV(a.dr64, k));
-      }
+      // vertical mass flux through half level k of the step: rho_ic ((1 - beta) w^n + beta w^{n+1})
+      const float fk = ri_k * ((float)(1.0 - kBeta) * wf_k + (float)kBeta * wnf);
+      const double t = fma(cd[LD_IDZ * ld + k], f32_to_f64(fk) - f32_to_f64(fflux_next), LMV(a.dr64, k));
       const double rho_n = rho_k - t;
       const float rho_nf = f64_to_f32(rho_n);
       const double thv_n = thv_k + f32_to_f64(__fdividef(dTh + f64_to_f32(t) * thv_kf, rho_nf));
@@ -1755,62 +1698,14 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
   }
   (void)wn_next;
   if (act) {
-    if constexpr (TOPO) {                            // the ground: the stage's terrain-following w
-      const float wg = a.t_wcc[o + N];
-      a.w32[o + N] = wg;
-      if (CORR) LMV(a.w, N) = f32_to_f64(wg);
-    } else {
-      a.w32[o + N] = 0.0f;
-      if (CORR) LMV(a.w, N) = 0.0;                   // the ground (w^n there is 0 already)
-    }
+    a.w32[cc * ld + N] = 0.0f;
+    if (CORR) LMV(a.w, N) = 0.0;                   // the ground (w^n there is 0 already)
   }
   if (!ok && act) atomicOr(a.status, 1u);
 #undef LMV
 }
 
-template <bool CORR, int U, int CH, int THREADS, int MINB, bool TOPO = false>
-__global__ void __launch_bounds__(THREADS, MINB) k_mx_lean_column(MxGeo G, MxLeanArgs a) {
-  __shared__ LeanTile<CH> T[THREADS / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t c0 = (int64_t)blockIdx.x * THREADS + warp * 32;
-  if (c0 >= G.nc) return;                            // whole warp past the end
-  mx_lean_column_item<CORR, U, CH, TOPO>(G, a, c0 + lane, c0, lane, T[warp]);
-}
-
-// launch shapes of the lean column, one thread per column in blocks of four warps: the tile's
-// "lanes" is the unroll factor of the two sweeps and its "block" the resident blocks per SM
-// the registers are held to (6: 80 registers, 8: 64, 9: 56, 10: 48, 12: 40). Only the register
-// cap varies among the candidates: it leaves the arithmetic as it is, while another unroll factor
-// changes which multiply-adds the compiler fuses and with them the FP32 roundings (measured:
-// unroll 1 or 4 moves vn by 1e-7 relative after one step), and a tuner choosing by timing
-// must not change results. The kernel waits on memory latency and gains from occupancy (12.2 ms
-// per R2B6/90 step at 10 blocks against 16.9 ms with 64-thread blocks at 94 registers); the
-// default, 9 blocks (36 warps per SM, 56 registers, no spills), measured 11.21 against 11.68 ms
-// at 10 blocks (48 registers, spilling in the corrector) and 161.3 against 162.4 ms at R2B8/90.
-const TileChoice kLeanShapes[] = {{2, 9}, {2, 10}, {2, 8}, {2, 12}, {2, 6}};
-const TileChoice kLeanDefault = {2, 9};
-
-bool lean_shape_ok(const TileChoice& t) {
-  for (const TileChoice& c : kLeanShapes)
-    if (c.lanes == t.lanes && c.block == t.block) return true;
-  return false;
-}
-
-template <bool CORR, bool TOPO = false>
-void launch_lean_column_as(const MxGeo& G, const MxLeanArgs& a, const TileChoice& t, cudaStream_t st) {
-  const unsigned nb = blocks_for(G.nc, 128);
-  if (t.block == 8) k_mx_lean_column<CORR, 2, 8, 128, 8, TOPO><<<nb, 128, 0, st>>>(G, a);
-  else if (t.block == 10) k_mx_lean_column<CORR, 2, 8, 128, 10, TOPO><<<nb, 128, 0, st>>>(G, a);
-  else if (t.block == 12) k_mx_lean_column<CORR, 2, 8, 128, 12, TOPO><<<nb, 128, 0, st>>>(G, a);
-  else if (t.block == 6) k_mx_lean_column<CORR, 2, 8, 128, 6, TOPO><<<nb, 128, 0, st>>>(G, a);
-  else k_mx_lean_column<CORR, 2, 8, 128, 9, TOPO><<<nb, 128, 0, st>>>(G, a);
-}
-
-template <bool CORR>
-void launch_lean_column(const MxGeo& G, const MxLeanArgs& a, const TileChoice& t, bool topo, cudaStream_t st) {
-  if (topo) launch_lean_column_as<CORR, true>(G, a, t, st);
-  else launch_lean_column_as<CORR, false>(G, a, t, st);
-}
+#include "lean_column.h"
 
 MxGeo make_mx_geo(const icon_grid* grid, const StateDev& s) {
   const GridDev& g = grid->g;
@@ -1999,11 +1894,6 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
       });
       break;
     }
-    case K_MX_LEAN: {          // the predictor's lean column (writes only the stage's scratch and S*)
-      const MxLeanArgs la = lean_args(s, false, (double)ea.dtau, 1);
-      launch_lean_column<false>(G, la, t, s.topo.on, st);
-      break;
-    }
     case K_MX_DIFF_EDGE:
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
@@ -2041,13 +1931,12 @@ void launch_mx_column(const MxGeo& G, const MxColArgs& a, bool topo, cudaStream_
 // ---------------------------------------------------------------- autotuner
 // Candidate tiles over (entity, level): 32 lanes per entity (one entity per warp), 16
 // (two per warp) or 8 (four per warp), blocks of 64, 128, 256 or 512 threads: twelve per
-// stencil kind. The lean column (one thread per column) chooses among its precompiled
-// launch shapes (kLeanShapes). Each kind is timed on the state's own data (three launches
+// stencil kind. (The lean column's form follows a rule on the grid's size, lean_form.) Each kind is timed on the state's own data (three launches
 // per candidate after one untimed, CUDA events) and the fastest kept, in the order of the
 // step, so that every trial reads inputs its predecessors formed. Choices are cached per
 // (kind, grid size, levels, GPU) in the process and, if the environment variable
 // ICON_TUNE_CACHE names a file, in that file.
-const int kTunedKinds[] = {K_MX_VERTEX, K_MX_EDGE, K_MX_CELL_KE, K_MX_EDGE_TEND, K_MX_COLUMN_PREP, K_MX_LEAN,
+const int kTunedKinds[] = {K_MX_VERTEX, K_MX_EDGE, K_MX_CELL_KE, K_MX_EDGE_TEND, K_MX_COLUMN_PREP,
                            K_MX_DIFF_VERTEX};
 const int kTileLanes[] = {32, 16, 8};
 const int kTileBlocks[] = {128, 256, 512, 64};
@@ -2090,7 +1979,7 @@ void save_tune_entry(const std::string& key, const TileChoice& t) {
 
 }  // namespace
 
-bool lean_column_shape_ok(int unroll, int blocks_per_sm) { return lean_shape_ok(TileChoice{unroll, blocks_per_sm}); }
+bool lean_column_shape_ok(int lanes, int form) { return lean_shape_ok(TileChoice{lanes, form}); }
 
 void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   StateDev& s = st->s;
@@ -2101,9 +1990,7 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   const MxColArgs ca = col_args(s, false, dtau, nsub);
   const bool lean = s.ln_B != nullptr;
   if (lean) {
-    // the lean gather's weights and the column's per-level constants for this dtau, so that
-    // the gather and column trials compute on valid inputs
-    k_mx_leanconst<<<1, 128, 0, stream>>>(G.N, G.ld, G.wu, G.wl, G.dzh, G.dz, G.ray, s.ex_ref, dtau, s.ln_cd, s.ln_cf);
+    // the lean gather's weights for this dtau, so that its trials compute on valid inputs
     k_mx_dwa_t<<<blocks_for(G.nc, 256), 256, 0, stream>>>(G.nc, G.div_wa, G.inv_Ac, dtau, s.ln_dwa, s.ln_cw32);
   }
   std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -2111,7 +1998,6 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   for (int kind : kTunedKinds) {
     if (st->tile[kind].lanes != 0 && st->tile_forced[kind]) continue;
     if (kind == K_MX_COLUMN_PREP && !s.fac64 && !lean) continue;
-    if (kind == K_MX_LEAN && !lean) continue;
     const std::string key = tune_key(kind, G);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
@@ -2119,12 +2005,8 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
       continue;
     }
     std::vector<TileChoice> cands;
-    if (kind == K_MX_LEAN) {
-      for (const TileChoice& c : kLeanShapes) cands.push_back(c);
-    } else {
-      for (int lanes : kTileLanes)
-        for (int block : kTileBlocks) cands.push_back(TileChoice{lanes, block});
-    }
+    for (int lanes : kTileLanes)
+      for (int block : kTileBlocks) cands.push_back(TileChoice{lanes, block});
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -2149,6 +2031,7 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   // a trial that met a non-finite value would have flagged the state; the step that
   // follows checks it again
   cudaMemsetAsync(s.status, 0, sizeof(unsigned), stream);
+  if (lean && !st->tile_forced[K_MX_LEAN]) st->tile[K_MX_LEAN] = kLeanDefault;
   st->tuned = true;
 }
 
@@ -2263,12 +2146,8 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
         prof_end(stream);
         if (overlap && (!corr || it + 1 < nsub)) fork_diag(!corr);
         prof_begin(stream, K_MX_LEAN);
-        // the autotuner times the predictor's column (the corrector updates S^n in place and
-        // cannot be run again on the state); the corrector, whose extra live values spill at
-        // 48 registers, keeps the default shape (56 registers, no spills) unless one is forced
         const TileChoice tc = st->tile[K_MX_LEAN].lanes ? st->tile[K_MX_LEAN] : kLeanDefault;
-        const TileChoice tcc = st->tile_forced[K_MX_LEAN] ? tc : kLeanDefault;
-        if (corr) launch_lean_column<true>(G, la, tcc, s.topo.on, stream);
+        if (corr) launch_lean_column<true>(G, la, tc, s.topo.on, stream);
         else launch_lean_column<false>(G, la, tc, s.topo.on, stream);
         prof_end(stream);
         continue;
