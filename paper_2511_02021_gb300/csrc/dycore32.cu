@@ -153,21 +153,17 @@ struct MxEdgeArgs {
 // group holds half level h = base + l and, except the last lane, full level k = h;
 // each half-level interpolant and cell-pair sum of w is formed once and passed to the
 // lane below with a shuffle (only the group's own lanes take part, so the two halves
-// of a warp may serve different entities). TOPO (terrain-following levels): per-edge
-// interpolation weights, w - wcc in the vertical advection, the metric correction of the
-// pressure gradient (exp is then against the per-cell reference), fluxes through dz_e.
-// HOIST: read the arguments the level loop uses once, the outputs through restrict pointers
-// (the per-state kernels: 5.6 -> 5.3 ms per R2B6/90 mixed step); the persistent ensemble
-// keeps them in its shared-memory slot and reads them there, which its 64-register budget
-// takes better (hoisted, its edge phase spilled and slowed from 55 to 79 ms per step)
-template <int LPE, bool TOPO = false, bool HOIST = true>
+// of a warp may serve different entities).
+// The persistent ensemble's form: it keeps its arguments in its shared-memory slot and reads
+// them there, which its 64-register budget takes better than holding them (hoisted, its edge
+// phase spilled and slowed from 55 to 79 ms per step).
+template <int LPE>
 __device__ inline void mx_edge_tend_item(const MxGeo& G, const MxEdgeArgs& a, int64_t e, int lane) {
   const int ld = G.ld, N = G.N;
   const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
   const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
   const float ide = G.inv_de32[e], ile = G.inv_le32[e], fe = G.f_e32[e], le = G.l_e32[e];
   const float cide = (float)kCpd * ide;
-  const float csn = TOPO ? a.t_csn[e] : 0.0f;
   const int64_t o = e * ld;
   const float* __restrict__ vn = a.vn + o;
   const float* __restrict__ vt = a.vt + o;
@@ -178,21 +174,6 @@ __device__ inline void mx_edge_tend_item(const MxGeo& G, const MxEdgeArgs& a, in
   const float* __restrict__ thv = a.thv;
   const float* __restrict__ exq = a.exp;
   const float* __restrict__ rho = a.rho;
-  // the arguments the level loop uses (vn_base, Avn0 and vn_out may be one buffer, updated
-  // element by element)
-  const float* __restrict__ wu32 = G.wu32;
-  const float* __restrict__ wl32 = G.wl32;
-  const float* __restrict__ idz32 = G.inv_dz32;
-  float* __restrict__ ae_o = a.a_e + o;
-  const float* vnb_o = a.vn_base + o;
-  float* avn_o = a.Avn0 + o;
-  float* vout_o = a.vn_out + o;
-  float* __restrict__ phi_o = a.phi + o;
-  float* __restrict__ gth_o = a.gth + o;
-  double* __restrict__ mflx_o = a.mflx + o;
-  const bool corr = a.corrector != 0, skip = a.skip_flux != 0, upw = a.upwind_theta != 0;
-  const float dtau = a.dtau;
-  const double inv_nsub = a.inv_nsub;
   static_assert(LPE == 8 || LPE == 16 || LPE == 32, "lane groups of 8, 16 or 32");
   const unsigned seg = LPE == 32 ? 0xffffffffu : (((1u << LPE) - 1u) << (threadIdx.x & (32 - LPE)));
 #pragma unroll 2   // two windows' loads in flight (the kernel is bound by load latency)
@@ -202,73 +183,43 @@ __device__ inline void mx_edge_tend_item(const MxGeo& G, const MxEdgeArgs& a, in
     const int hl = h > 0 ? (h - 1 < N - 1 ? h - 1 : N - 1) : 0;
     const int hu = h < N ? h : N - 1;
     const bool inner = h > 0 && h < N;
-    float wa, wb;
-    if constexpr (TOPO) {
-      wa = inner ? a.t_wu_e[o + h] : (h == 0 ? 0.0f : 1.0f);
-      wb = inner ? 1.0f - wa : (h == 0 ? 1.0f : 0.0f);
-    } else {
-      wa = inner ? (HOIST ? wu32 : G.wu32)[h] : (h == 0 ? 0.0f : 1.0f);
-      wb = inner ? (HOIST ? wl32 : G.wl32)[h] : (h == 0 ? 1.0f : 0.0f);
-    }
+    const float wa = inner ? G.wu32[h] : (h == 0 ? 0.0f : 1.0f);
+    const float wb = inner ? G.wl32[h] : (h == 0 ? 1.0f : 0.0f);
     float vie = 0.f, tie = 0.f, sw = 0.f, dw = 0.f, dwv = 0.f;
     if (hv) {
       vie = wa * vn[hl] + wb * vn[hu];
       tie = wa * vt[hl] + wb * vt[hu];
       const float w1 = w[c1 + h], w2 = w[c2 + h];
-      if constexpr (TOPO) sw = a.t_wcon[c1 + h] + a.t_wcon[c2 + h];     // 0 at the lid and the ground
-      else sw = w1 + w2;
+      sw = w1 + w2;
       dw = w2 - w1;
       dwv = wv[v2 + h] - wv[v1 + h];
     }
     const float vie_up = __shfl_down_sync(seg, vie, 1, LPE);
     const float sw_up = __shfl_down_sync(seg, sw, 1, LPE);
     if (!hv || lane == LPE - 1) continue;
-    if constexpr (HOIST) ae_o[h] = vie * dw * ide + tie * dwv * ile;
-    else a.a_e[o + h] = vie * dw * ide + tie * dwv * ile;
+    a.a_e[o + h] = vie * dw * ide + tie * dwv * ile;
     if (h == N) continue;
     const int k = h;
     const float wbar = 0.25f * (sw + sw_up);
     const float zeta_e = 0.5f * (zeta[v1 + k] + zeta[v2 + k]);
     const float A = -(Kc[c2 + k] - Kc[c1 + k]) * ide + (zeta_e + fe) * vt[k] -
-                    wbar * (vie - vie_up) * (TOPO ? a.t_inv_dz_e[o + k] : (HOIST ? idz32 : G.inv_dz32)[k]);
+                    wbar * (vie - vie_up) * G.inv_dz32[k];
     const float t1 = thv[c1 + k], t2 = thv[c2 + k];
     const float th_e = 0.5f * (t1 + t2);
-    float pg;
-    if constexpr (TOPO)
-      pg = th_e * ((exq[c2 + k] - exq[c1 + k]) * cide - (csn * a.t_bf[k]) * (a.t_hdpdz[c1 + k] + a.t_hdpdz[c2 + k]));
-    else
-      pg = th_e * ((exq[c2 + k] - exq[c1 + k]) * cide);
+    const float pg = th_e * ((exq[c2 + k] - exq[c1 + k]) * cide);
     float vnew;
-    if constexpr (HOIST) {
-      if (corr) {
-        vnew = vnb_o[k] + dtau * (0.5f * (avn_o[k] + A) - pg);
-      } else {
-        vnew = vnb_o[k] + dtau * (A - pg);
-        avn_o[k] = A;
-      }
-      vout_o[k] = vnew;
-      if (skip) continue;
+    if (a.corrector) {
+      vnew = a.vn_base[o + k] + a.dtau * (0.5f * (a.Avn0[o + k] + A) - pg);
     } else {
-      if (a.corrector) {
-        vnew = a.vn_base[o + k] + a.dtau * (0.5f * (a.Avn0[o + k] + A) - pg);
-      } else {
-        vnew = a.vn_base[o + k] + a.dtau * (A - pg);
-        a.Avn0[o + k] = A;
-      }
-      a.vn_out[o + k] = vnew;
-      if (a.skip_flux) continue;
+      vnew = a.vn_base[o + k] + a.dtau * (A - pg);
+      a.Avn0[o + k] = A;
     }
-    float F = 0.5f * (rho[c1 + k] + rho[c2 + k]) * vnew;
-    if constexpr (TOPO) F *= a.t_dz_e[o + k];
-    if constexpr (HOIST) {
-      phi_o[k] = F;
-      gth_o[k] = (le * F) * (upw ? (vnew >= 0.0f ? t1 : t2) : th_e);
-      if (corr) mflx_o[k] += f32_to_f64(F) * inv_nsub;
-    } else {
-      a.phi[o + k] = F;
-      a.gth[o + k] = (le * F) * (a.upwind_theta ? (vnew >= 0.0f ? t1 : t2) : th_e);
-      if (a.corrector) a.mflx[o + k] += f32_to_f64(F) * a.inv_nsub;
-    }
+    a.vn_out[o + k] = vnew;
+    if (a.skip_flux) continue;
+    const float F = 0.5f * (rho[c1 + k] + rho[c2 + k]) * vnew;
+    a.phi[o + k] = F;
+    a.gth[o + k] = (le * F) * (a.upwind_theta ? (vnew >= 0.0f ? t1 : t2) : th_e);
+    if (a.corrector) a.mflx[o + k] += f32_to_f64(F) * a.inv_nsub;
   }
 }
 
@@ -287,11 +238,6 @@ __device__ inline void mx_dd_div_item(const MxGeo& G, const float* __restrict__ 
   for (int k = lane; k < G.N; k += 32) D[c * ld + k] = dw[0] * vn[E[0] + k] + dw[1] * vn[E[1] + k] + dw[2] * vn[E[2] + k];
 }
 
-__global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restrict__ vn, float* __restrict__ D) {
-  const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (c < G.nc) mx_dd_div_item(G, vn, D, c, threadIdx.x & 31);
-}
-
 __device__ inline void mx_dd_lap_item(const MxGeo& G, const float* __restrict__ D, float* __restrict__ L, int64_t c,
                                       int lane) {
   const int ld = G.ld;
@@ -306,11 +252,6 @@ __device__ inline void mx_dd_lap_item(const MxGeo& G, const float* __restrict__ 
   for (int k = lane; k < G.N; k += 32)
     L[c * ld + k] = wt[0] * (D[B[0] + k] - D[A[0] + k]) + wt[1] * (D[B[1] + k] - D[A[1] + k]) +
                     wt[2] * (D[B[2] + k] - D[A[2] + k]);
-}
-
-__global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restrict__ D, float* __restrict__ L) {
-  const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (c < G.nc) mx_dd_lap_item(G, D, L, c, threadIdx.x & 31);
 }
 
 struct MxDDArgs {
@@ -393,8 +334,7 @@ __device__ inline void mx_diff_edge_item(const MxGeo& G, float* __restrict__ vn,
                                          const float* __restrict__ uy, const float* __restrict__ uz,
                                          const float* __restrict__ zeta, const float* __restrict__ divc,
                                          const float* __restrict__ thv, float* __restrict__ thflx, float dt, int64_t e,
-                                         int lane, const float* __restrict__ D1 = nullptr,
-                                         const float* __restrict__ zeta1 = nullptr, float bd_scale = 0.0f) {
+                                         int lane) {
   const int ld = G.ld;
   int64_t Q[4];
   for (int j = 0; j < 4; ++j) Q[j] = (int64_t)G.e2q[4 * e + j] * ld;
@@ -411,12 +351,7 @@ __device__ inline void mx_diff_edge_item(const MxGeo& G, float* __restrict__ vn,
     const float DS = (ax * tx + ay * ty + az * tz) * i34 + (bx * nx + by * ny + bz * nz) * ile;
     const float Kh = cs2ld * sqrtf(DT * DT + DS * DS);
     const float lap = (divc[c2 + k] - divc[c1 + k]) * ide - (zeta[v2 + k] - zeta[v1 + k]) * ile;
-    float vnew = vn[e * ld + k] + dt * Kh * lap;
-    if (D1) {                              // fourth-order background diffusion (option)
-      const float lap2 = (D1[c2 + k] - D1[c1 + k]) * ide - (zeta1[v2 + k] - zeta1[v1 + k]) * ile;
-      vnew -= bd_scale * lap2;
-    }
-    vn[e * ld + k] = vnew;
+    vn[e * ld + k] = vn[e * ld + k] + dt * Kh * lap;
     thflx[e * ld + k] = le * Kh * (thv[c2 + k] - thv[c1 + k]) * ide;
   }
 }
@@ -924,10 +859,9 @@ __device__ inline void mx_column_any(const MxGeo& G, const MxColArgs& a, int64_t
 
 // diffusion of theta_v for one column: FP32 increment, FP64 accumulation, Exner at
 // constant density, shadows refreshed
-// (exref_c: the per-cell reference of terrain-following levels, [Nc][ld], or NULL)
 __device__ inline void mx_diff_theta_item(const MxGeo& G, const float* __restrict__ thflx, double* __restrict__ thv,
                                           double* __restrict__ ex, float* __restrict__ thv32, float* __restrict__ exp32,
-                                          float dt, int64_t c, const double* __restrict__ exref_c = nullptr) {
+                                          float dt, int64_t c) {
   const int64_t nc = G.nc;
   const int ld = G.ld;
   int64_t E[3];
@@ -946,56 +880,12 @@ __device__ inline void mx_diff_theta_item(const MxGeo& G, const float* __restric
     thv[i] = th_n;
     ex[i] = ex_n;
     thv32[c * ld + k] = f64_to_f32(th_n);
-    exp32[c * ld + k] = f64_to_f32(ex_n - (exref_c ? exref_c[c * ld + k] : G.ex_ref[k]));
+    exp32[c * ld + k] = f64_to_f32(ex_n - G.ex_ref[k]);
   }
 }
 
-// ---------------------------------------------------------------- per-state kernels
+// ---------------------------------------------------------------- stored-factor column, per state
 
-// warp w, lanes [sub*LPE, (sub+1)*LPE) handle entity w * (32/LPE) + sub
-#define ITEM_PROLOGUE(LPE, COUNT)                                                        \
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;             \
-  const int64_t item = gw * (32 / (LPE)) + (int64_t)((threadIdx.x & 31) / (LPE));        \
-  const int lane = (int)(threadIdx.x & ((LPE) - 1));                                     \
-  if (item >= (COUNT)) return;
-
-template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_vertex(MxGeo G, const float* vn, const float* w, float* zeta, float* w_v) {
-  ITEM_PROLOGUE(LPE, G.nv)
-  mx_vertex_item<LPE>(G, vn, w, zeta, w_v, item, lane);
-}
-template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_edge_diag(MxGeo G, const float* vn, float* vt) {
-  ITEM_PROLOGUE(LPE, G.ne)
-  mx_edge_diag_item<LPE>(G, vn, vt, item, lane);
-}
-template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_cell_ke(MxGeo G, const float* vn, const float* vt, float* Kc) {
-  ITEM_PROLOGUE(LPE, G.nc)
-  mx_cell_ke_item<LPE>(G, vn, vt, Kc, item, lane);
-}
-template <int LPE, bool TOPO = false>
-__global__ void __launch_bounds__(512, 2) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
-  ITEM_PROLOGUE(LPE, G.ne)
-  mx_edge_tend_item<LPE, TOPO>(G, a, item, lane);
-}
-template <int LPE>
-__global__ void __launch_bounds__(512, 2) k_mx_diff_vertex(MxGeo G, const float* vn, float* ux, float* uy, float* uz,
-                                                        float* zeta, float* divc) {
-  // vertices first, then cells (divergence): both only read vn
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t item = gw * (32 / LPE) + (int64_t)((threadIdx.x & 31) / LPE);
-  const int lane = (int)(threadIdx.x & (LPE - 1));
-  if (item < G.nv) mx_diff_vertex_item<LPE>(G, vn, ux, uy, uz, zeta, item, lane);
-  else if (item < G.nv + G.nc) mx_diff_div_item<LPE>(G, vn, divc, item - G.nv, lane);
-}
-template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_diff_edge(MxGeo G, float* vn, const float* ux, const float* uy,
-                                                      const float* uz, const float* zeta, const float* divc,
-                                                      const float* thv, float* thflx, float dt) {
-  ITEM_PROLOGUE(LPE, G.ne)
-  mx_diff_edge_item<LPE>(G, vn, ux, uy, uz, zeta, divc, thv, thflx, dt, item, lane);
-}
 // Gather step of the stored-factor column path for one state: a block takes 32
 // consecutive cells and walks the levels in chunks of LPE; lane groups of LPE
 // threads compute one cell's chunk (coalesced reads of its edge and cell rows), the
@@ -1079,16 +969,6 @@ __device__ inline void mx_gather_tile_body(const MxGeo& G, const MxColArgs& a, i
     }
     __syncthreads();
   }
-}
-
-// the diffusion edge step with fourth-order background diffusion (option): 32 lanes per edge
-__global__ void __launch_bounds__(256) k_mx_diff_edge_bd(MxGeo G, float* vn, const float* ux, const float* uy,
-                                                         const float* uz, const float* zeta, const float* divc,
-                                                         const float* thv, float* thflx, float dt, const float* D1,
-                                                         const float* zeta1, float bd_scale) {
-  const int64_t e = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (e >= G.ne) return;
-  mx_diff_edge_item<32>(G, vn, ux, uy, uz, zeta, divc, thv, thflx, dt, e, threadIdx.x & 31, D1, zeta1, bd_scale);
 }
 
 template <int LPE, bool CORR>
@@ -1236,12 +1116,6 @@ __global__ void __launch_bounds__(128) k_mx_column(MxGeo G, MxColArgs a) {
   if constexpr (TOPO) mx_column_item<NMAX, CORR, true>(G, a, c);     // always recomputes its factors
   else mx_column_any<NMAX, CORR>(G, a, c);
 }
-__global__ void __launch_bounds__(128) k_mx_diff_theta(MxGeo G, const float* thflx, double* thv, double* ex,
-                                                       float* thv32, float* exp32, float dt, const double* exref_c) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < G.nc) mx_diff_theta_item(G, thflx, thv, ex, thv32, exp32, dt, c, exref_c);
-}
-
 // ---------------------------------------------------------------- lean column (flat levels)
 //
 // The column of a mixed-precision state on flat levels in the fewest FP64 operations the
@@ -1338,17 +1212,14 @@ struct LeanTile {
 };
 
 // gather of the lean column's stage inputs for 32 consecutive cells: lanes over levels
-// (LPE per cell), transposed through shared memory into level-major rows
+// (LPE per cell), transposed through shared memory into level-major rows (the persistent ensemble's form)
 template <int LPE>
 struct LeanGatherTile {
   double d[LPE][kGatherCells + 1];
   float f[4][LPE][kGatherCells + 1];       // dtau D_Theta, dtau A_w, A_w (predictor), dtau D_rho (predictor)
 };
 
-// TOPO (terrain-following levels): the damped fluxes through the edges' layer thickness, the
-// vertical advection of w with w - wcc and the cell's own 1/dzh; the divergences stay per unit
-// thickness here and the column scales them by the cell's 1/dz
-template <int LPE, bool CORR, bool DDF = false, bool TOPO = false>
+template <int LPE, bool CORR, bool DDF = false>
 __device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, int64_t c0, LeanGatherTile<LPE>& T) {
   constexpr int CB = kGatherCells;
   const int N = G.N, ld = G.ld;
@@ -1401,7 +1272,6 @@ __device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, 
           for (int s = 0; s < 3; ++s) {
             const float vd = a.dd_vn[E[s] + k] - sc[s] * (a.dd_L[Cb[s] + k] - a.dd_L[Ca[s] + k]);
             F[s] = 0.5f * (a.dd_rho[Ca[s] + k] + a.dd_rho[Cb[s] + k]) * vd;
-            if constexpr (TOPO) F[s] *= a.t_dz_e[E[s] + k];
             const float t1 = a.dd_thv[Ca[s] + k], t2 = a.dd_thv[Cb[s] + k];
             Gt[s] = (le[s] * F[s]) * (a.dd_upwind ? (vd >= 0.0f ? t1 : t2) : 0.5f * (t1 + t2));
             if (own[s]) {
@@ -1423,11 +1293,7 @@ __device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, 
       }
       if (k >= 1 && k < N) {
         const float hadv = kw[0] * a.a_e[E[0] + k] + kw[1] * a.a_e[E[1] + k] + kw[2] * a.a_e[E[2] + k];
-        float Aw;
-        if constexpr (TOPO)
-          Aw = -hadv - a.t_wcon[o + k] * (a.w_stage[o + k - 1] - a.w_stage[o + k + 1]) * (0.5f * a.t_inv_dzh[o + k]);
-        else
-          Aw = -hadv - a.w_stage[o + k] * (a.w_stage[o + k - 1] - a.w_stage[o + k + 1]) * G.inv_dz2_32[k];
+        float Aw = -hadv - a.w_stage[o + k] * (a.w_stage[o + k - 1] - a.w_stage[o + k + 1]) * G.inv_dz2_32[k];
         if (CORR) Aw = 0.5f * (T.f[2][lane][cl] + Aw);
         else T.f[2][lane][cl] = Aw;
         T.f[1][lane][cl] = dtau32 * Aw;
@@ -1449,20 +1315,6 @@ __device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, 
     }
     __syncthreads();
   }
-}
-
-template <int LPE, bool CORR, bool DDF = false, bool TOPO = false>
-__global__ void __launch_bounds__(512, 3) k_mx_lean_gather(MxGeo G, MxLeanArgs a) {
-  __shared__ LeanGatherTile<LPE> T;
-  mx_lean_gather_body<LPE, CORR, DDF, TOPO>(G, a, (int64_t)blockIdx.x * kGatherCells, T);
-}
-
-// the corrector's gather with the damping fused in (32 lanes per cell, 256-thread blocks: the
-// fastest of six tiles measured at R2B6/90, within 13 % of one another)
-void launch_lean_gather_dd(const MxGeo& G, const MxLeanArgs& a, bool topo, cudaStream_t st) {
-  const unsigned nb = (unsigned)((G.nc + kGatherCells - 1) / kGatherCells);
-  if (topo) k_mx_lean_gather<32, true, true, true><<<nb, 256, 0, st>>>(G, a);
-  else k_mx_lean_gather<32, true, true><<<nb, 256, 0, st>>>(G, a);
 }
 
 // write the finished chunk [k0, k0 + CH) of the warp's 32 columns (first cell c0): CH lanes
@@ -1705,6 +1557,7 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
 #undef LMV
 }
 
+#include "stencils32.h"
 #include "lean_column.h"
 
 MxGeo make_mx_geo(const icon_grid* grid, const StateDev& s) {
@@ -1844,6 +1697,20 @@ void with_lanes(int lanes, F f) {
   else f(std::integral_constant<int, 32>{});
 }
 
+// the lean gather: blocks of at most 256 threads (32 groups of eight lanes, one per cell)
+template <bool CORR>
+void launch_lean_gather(const MxGeo& G, const MxLeanArgs& a, bool fused, bool topo, int block, cudaStream_t st) {
+  const unsigned nb = blocks_for(G.nc, 32);
+  const int B = block < 256 ? block : 256;
+  if (CORR && fused) {
+    if (topo) k_mx_lean_gather<CORR, CORR, true><<<nb, B, 0, st>>>(G, a);
+    else k_mx_lean_gather<CORR, CORR, false><<<nb, B, 0, st>>>(G, a);
+  } else {
+    if (topo) k_mx_lean_gather<CORR, false, true><<<nb, B, 0, st>>>(G, a);
+    else k_mx_lean_gather<CORR, false, false><<<nb, B, 0, st>>>(G, a);
+  }
+}
+
 void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, const MxEdgeArgs& ea,
                  const MxColArgs& ca, float dt, cudaStream_t st) {
   const int B = t.block;
@@ -1870,7 +1737,7 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
         if (s.topo.on) k_mx_edge_tend<LPE, true><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
-        else k_mx_edge_tend<LPE><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
+        else k_mx_edge_tend<LPE, false><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
       });
       break;
     case K_MX_DIFF_VERTEX:
@@ -1882,25 +1749,16 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
       break;
     case K_MX_COLUMN_PREP: {   // the predictor's gather (the corrector's only differs in the Aw0 average)
       const unsigned nb = (unsigned)((G.nc + 31) / 32);
+      if (s.ln_B) {
+        launch_lean_gather<false>(G, lean_args(s, false, (double)ea.dtau, 1), false, s.topo.on, B, st);
+        break;
+      }
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
-        if (s.ln_B) {
-          const MxLeanArgs la = lean_args(s, false, (double)ea.dtau, 1);
-          if (s.topo.on) k_mx_lean_gather<LPE, false, false, true><<<nb, B, 0, st>>>(G, la);
-          else k_mx_lean_gather<LPE, false><<<nb, B, 0, st>>>(G, la);
-        } else {
-          k_mx_gather_tile<LPE, false><<<nb, B, 0, st>>>(G, ca);
-        }
+        k_mx_gather_tile<LPE, false><<<nb, B, 0, st>>>(G, ca);
       });
       break;
     }
-    case K_MX_DIFF_EDGE:
-      with_lanes(t.lanes, [&](auto L) {
-        constexpr int LPE = decltype(L)::value;
-        k_mx_diff_edge<LPE><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, s.vn32, s.uvx32, s.uvy32, s.uvz32, s.zeta32,
-                                                                     s.Kc32, s.thv32, s.vt32, dt);
-      });
-      break;
     default: break;
   }
 }
@@ -2006,7 +1864,9 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
     }
     std::vector<TileChoice> cands;
     for (int lanes : kTileLanes)
-      for (int block : kTileBlocks) cands.push_back(TileChoice{lanes, block});
+      for (int block : kTileBlocks)
+        if (!(kind == K_MX_COLUMN_PREP && lean) || (lanes == 8 && block <= 256))   // the lean gather's lanes are fixed
+          cands.push_back(TileChoice{lanes, block});
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -2111,10 +1971,10 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
         da.vn = s.vn32; da.phi = s.F32; da.gth = s.G32; da.mflx = s.mflx;
         da.scale = (float)(st->divdamp4 * abar * abar); da.inv_nsub = 1.0 / nsub;
         da.upwind_theta = st->upwind_theta ? 1 : 0;
-        const unsigned nbc8 = (unsigned)((nc + 7) / 8), nbe8 = (unsigned)((G.ne + 7) / 8);
+        const unsigned nbq = item_blocks(nc, kQuadLanes, 256), nbe8 = (unsigned)((G.ne + 7) / 8);
         prof_begin(stream, K_DIVDAMP);
-        k_mx_dd_div<<<nbc8, 256, 0, stream>>>(G, fused ? s.Avn0_32 : s.vn32, s.Kc32);
-        k_mx_dd_lap<<<nbc8, 256, 0, stream>>>(G, s.Kc32, s.vt32);
+        k_mx_dd_div<<<nbq, 256, 0, stream>>>(G, fused ? s.Avn0_32 : s.vn32, s.Kc32);
+        k_mx_dd_lap<<<nbq, 256, 0, stream>>>(G, s.Kc32, s.vt32);
         if (!fused) k_mx_dd_edge<<<nbe8, 256, 0, stream>>>(G, da);
         prof_end(stream);
       }
@@ -2126,23 +1986,10 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
           la.dd_scale = (float)(st->divdamp4 * st->abar * st->abar);
           la.dd_upwind = st->upwind_theta ? 1 : 0;
         }
-        const TileChoice t = tile(K_MX_COLUMN_PREP);
-        const unsigned nb = (unsigned)((nc + 31) / 32);
+        const int block = tile(K_MX_COLUMN_PREP).block;
         prof_begin(stream, K_MX_LEAN_GATHER);
-        if (corr && fused) {
-          launch_lean_gather_dd(G, la, s.topo.on, stream);
-        } else {
-          with_lanes(t.lanes, [&](auto L) {
-            constexpr int LPE = decltype(L)::value;
-            if (s.topo.on) {
-              if (corr) k_mx_lean_gather<LPE, true, false, true><<<nb, t.block, 0, stream>>>(G, la);
-              else k_mx_lean_gather<LPE, false, false, true><<<nb, t.block, 0, stream>>>(G, la);
-            } else {
-              if (corr) k_mx_lean_gather<LPE, true><<<nb, t.block, 0, stream>>>(G, la);
-              else k_mx_lean_gather<LPE, false><<<nb, t.block, 0, stream>>>(G, la);
-            }
-          });
-        }
+        if (corr) launch_lean_gather<true>(G, la, fused, s.topo.on, block, stream);
+        else launch_lean_gather<false>(G, la, false, s.topo.on, block, stream);
         prof_end(stream);
         if (overlap && (!corr || it + 1 < nsub)) fork_diag(!corr);
         prof_begin(stream, K_MX_LEAN);
@@ -2176,24 +2023,20 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
   prof_end(stream);
   if (st->diff4 > 0.0) {
     // dead after the substeps: ae32 (edges) holds L(vn), w32_s its curl, exp32_s its divergence
-    const double abar = st->abar;
     prof_begin(stream, K_DIFF4);
     k_mx_bd_lap<<<(unsigned)((G.ne + 7) / 8), 256, 0, stream>>>(G, s.zeta32, s.Kc32, s.ae32);
     k_mx_bd_curldiv<<<(unsigned)((G.nv + nc + 7) / 8), 256, 0, stream>>>(G, s.ae32, s.w32_s, s.exp32_s);
     prof_end(stream);
-    prof_begin(stream, K_MX_DIFF_EDGE);
-    const unsigned nbe8 = (unsigned)((G.ne + 7) / 8);
-    k_mx_diff_edge_bd<<<nbe8, 256, 0, stream>>>(G, s.vn32, s.uvx32, s.uvy32, s.uvz32, s.zeta32, s.Kc32, s.thv32,
-                                                s.vt32, (float)dt, s.exp32_s, s.w32_s, (float)(st->diff4 * abar * abar));
-    prof_end(stream);
-  } else {
-    prof_begin(stream, K_MX_DIFF_EDGE);
-    launch_kind(K_MX_DIFF_EDGE, tile(K_MX_DIFF_EDGE), G, s, ea, ca, (float)dt, stream);
-    prof_end(stream);
   }
+  const bool bd = st->diff4 > 0.0;
+  prof_begin(stream, K_MX_DIFF_EDGE);
+  k_mx_diff_edge<<<item_blocks(G.ne, kQuadLanes, 256), 256, 0, stream>>>(
+      G, s.vn32, s.uvx32, s.uvy32, s.uvz32, s.zeta32, s.Kc32, s.thv32, s.vt32, (float)dt, bd ? s.exp32_s : nullptr,
+      bd ? s.w32_s : nullptr, (float)(st->diff4 * st->abar * st->abar));
+  prof_end(stream);
   prof_begin(stream, K_MX_DIFF_THETA);
-  k_mx_diff_theta<<<blocks_for(nc, 128), 128, 0, stream>>>(G, s.vt32, s.thv, s.ex, s.thv32, s.exp32, (float)dt,
-                                                           s.topo.on ? s.topo.exref_c : nullptr);
+  k_mx_diff_theta<<<blocks_for(nc, 32), 256, 0, stream>>>(G, s.vt32, s.thv, s.ex, s.thv32, s.exp32, (float)dt,
+                                                          s.topo.on ? s.topo.exref_lm : nullptr);
   prof_end(stream);
 }
 
@@ -2588,9 +2431,9 @@ __global__ void __launch_bounds__(128, MINB) k_ensemble_step(EnsArgs A) {
       warp_pairs<kChunk>(
           s_off_e, A.nm, A.tot_e, gwarp, nwarps,
           [&](int m, int64_t j) {
-            mx_edge_tend_item<16, false, false>(geo(m), edge_args_of(m, stage), j + (lane >> 4), lane & 15);
+            mx_edge_tend_item<16>(geo(m), edge_args_of(m, stage), j + (lane >> 4), lane & 15);
           },
-          [&](int m, int64_t j) { mx_edge_tend_item<32, false, false>(geo(m), edge_args_of(m, stage), j, lane); });
+          [&](int m, int64_t j) { mx_edge_tend_item<32>(geo(m), edge_args_of(m, stage), j, lane); });
       if (!sync(ICON_ENS_PH_EDGE_TEND)) return;
       if (stage == 1 && A.any_damp) {
         // divergence damping of vn^{n+1}: cell divergence (into Kc32), its Laplacian (into
