@@ -248,14 +248,16 @@ int alloc_state(icon_state* st, int precision, bool topo) {
     double** col[] = {&s.col_lo, &s.col_di, &s.col_up, &s.col_rh, &s.col_rx,
                       &s.col_tx, &s.col_px, &s.col_gm, &s.col_ri, &s.col_mm, &s.col_ws, &s.col_gc};
     for (double** p : col) *p = A.get_n<double>(C);
+    if (!topo) s.col_d0 = A.get_n<double>(C);
     s.vn = A.get_n<double>(E); s.vn_s = A.get_n<double>(E);
     s.Avn0 = A.get_n<double>(E); s.Aw0 = A.get_n<double>(C);
     s.zeta = A.get_n<double>(V); s.w_v = A.get_n<double>(V);
     s.vt = A.get_n<double>(E); s.Ke = A.get_n<double>(E); s.Kc = A.get_n<double>(C);
     s.a_e = A.get_n<double>(E); s.F = A.get_n<double>(E); s.G = A.get_n<double>(E);
     s.kin_w_h = A.get_n<double>(3 * (size_t)nc); s.div_wa_h = A.get_n<double>(3 * (size_t)nc);
+    s.adv_w = A.get_n<double>(3 * (size_t)nc);
     // diffusion scratch reuses substep scratch (they never overlap in time)
-    s.Kh = s.vt; s.thflx = s.Ke; s.divc = s.Kc; s.uvx = s.w_v;
+    s.thflx = s.Ke; s.divc = s.Kc; s.uvx = s.w_v;
     s.uvy = A.get_n<double>(V); s.uvz = A.get_n<double>(V);
   } else {
     // FP64 prognostics level-major [k][Nc]; everything the stencils touch is FP32 [entity][ld]

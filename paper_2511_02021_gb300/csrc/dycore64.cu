@@ -56,6 +56,7 @@ struct Geo64 {
   const double *wu, *wl, *inv_dz, *inv_dz2, *qinv_dz;
   const double* cc;                        // per-level constants for the current dtau
   const double *kin_w_h, *div_wa_h;        // half the cell weights (state tables, [Nc][3])
+  const double* adv_w;                     // kappa_ce / d_e (state table, [Nc][3]): w advection
   // terrain-following levels (the TOPO kernel variants; see terrain.cu): per-edge normal
   // slope factor, full-level decay, per-entity tables [entity][ld], and the stage's
   // contravariant correction, contravariant velocity, Exner perturbation and half its
@@ -64,10 +65,9 @@ struct Geo64 {
   const double *t_wu_c, *t_inv_dz_c, *t_inv_dzh_c, *t_wcc, *t_wcon, *t_ep, *t_hdpdz;
 };
 
-// per-level constants of the column solve for one dtau, [8][ld] (same layout as the
-// mixed path): wu, wl, dtau beta cpd / dzh, (1 - beta) cpd / dzh, 1/(1 + dtau r),
-// dtau beta / dz, dtau (1 - beta) / dz, unused
-enum { C_WU = 0, C_WL, C_CA, C_CX, C_DAMP, C_DTBDZ, C_DT1BDZ, C_COUNT };
+// per-level constants of the column solve for one dtau, [8][ld]: wu, wl, dtau beta cpd / dzh,
+// cpd / dzh, 1/(1 + dtau r), dtau beta / dz, dtau (1 - beta) / dz, 2 beta / dz
+enum { C_WU = 0, C_WL, C_CA, C_CX, C_DAMP, C_DTBDZ, C_DT1BDZ, C_2BDZ, C_COUNT };
 
 __global__ void k_colconst64(int N, int ld, const double* __restrict__ wu, const double* __restrict__ wl,
                              const double* __restrict__ dzh, const double* __restrict__ dz,
@@ -77,10 +77,11 @@ __global__ void k_colconst64(int N, int ld, const double* __restrict__ wu, const
     cc[C_WU * ld + i] = i <= N ? wu[i] : 0.0;
     cc[C_WL * ld + i] = i <= N ? wl[i] : 0.0;
     cc[C_CA * ld + i] = interior ? dtau * kBeta * kCpd / dzh[i] : 0.0;
-    cc[C_CX * ld + i] = interior ? (1.0 - kBeta) * kCpd / dzh[i] : 0.0;
+    cc[C_CX * ld + i] = interior ? kCpd / dzh[i] : 0.0;
     cc[C_DAMP * ld + i] = i <= N ? 1.0 / (1.0 + dtau * ray[i]) : 1.0;
     cc[C_DTBDZ * ld + i] = i < N ? dtau * kBeta / dz[i] : 0.0;
     cc[C_DT1BDZ * ld + i] = i < N ? dtau * (1.0 - kBeta) / dz[i] : 0.0;
+    cc[C_2BDZ * ld + i] = i < N ? 2.0 * kBeta / dz[i] : 0.0;
   }
 }
 
@@ -97,7 +98,8 @@ __device__ inline int64_t warp_entity() {
   return (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
 }
 
-// zeta_v (full levels) and w_v (half levels)
+// zeta_v (full levels) and six times w_v (half levels): the plain sum of a hexagon's cells,
+// scaled by 6/5 at the twelve pentagons (the 1/6 is in the edge tendency's per-edge constant)
 __global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __restrict__ vn, const double* __restrict__ w,
                                                 double* __restrict__ zeta, double* __restrict__ w_v) {
   const int64_t v = warp_entity();
@@ -110,8 +112,7 @@ __global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __rest
     C[j] = (int64_t)G.v2c[6 * v + j] * ld;
     rw[j] = G.rot_wa[6 * v + j];
   }
-  const int deg = G.vdeg[v];
-  const double inv_deg = deg == 6 ? 1.0 / 6.0 : 1.0 / 5.0;
+  const bool penta = G.vdeg[v] != 6;
   for (int k = lane; k < G.N; k += 32) {
     double acc = 0.0;
     for (int j = 0; j < 6; ++j) acc += rw[j] * vn[E[j] + k];
@@ -120,8 +121,9 @@ __global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __rest
   for (int h = lane; h <= G.N; h += 32) {
     double acc = 0.0;
     for (int j = 0; j < 5; ++j) acc += w[C[j] + h];
-    acc += (deg == 6) ? w[C[5] + h] : 0.0;
-    w_v[v * ld + h] = acc * inv_deg;
+    if (penta) acc *= 1.2;
+    else acc += w[C[5] + h];
+    w_v[v * ld + h] = acc;
   }
 }
 
@@ -200,7 +202,9 @@ __global__ void __launch_bounds__(256, 4) k_edge_tend(Geo64 G, EdgeArgs a) {
   const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
   const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
   const int64_t eo = e * ld;
-  const double ide = G.inv_de[e], ile = G.inv_le[e], fe = G.f_e[e];
+  const double ide = G.inv_de[e], fe = G.f_e[e];
+  // a_e is stored times d_e (the cells' weights carry 1/d_e); w_v is six times the mean
+  const double rt = (G.inv_le[e] * G.d_e[e]) * (1.0 / 6.0);
   // the factors 1/2 of theta_e = (t1 + t2)/2 and rho_e = (rho1 + rho2)/2 are folded into
   // these constants (and the column's divergence weights), exact scalings by powers of two
   const double hcide = 0.5 * (kCpd * ide);
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(256, 4) k_edge_tend(Geo64 G, EdgeArgs a) {
     }
     const double vie_up = __shfl_down_sync(0xffffffffu, vie, 1);   // half level h + 1
     const double sw_up = __shfl_down_sync(0xffffffffu, sw, 1);
-    if (hv && lane < 31) a.a_e[eo + h] = (vie * dw) * ide + (tie * dwv) * ile;
+    if (hv && lane < 31) a.a_e[eo + h] = fma(vie, dw, (tie * rt) * dwv);
     if (kv) {
       const int k = h;
       // advective tendency: -grad K + (zeta + f) vt - wbar dvn/dz, with
@@ -306,17 +310,18 @@ __global__ void __launch_bounds__(256, 4) k_dd_lap(Geo64 G, const double* __rest
   const int64_t c = warp_entity();
   if (c >= G.nc) return;
   const int lane = threadIdx.x & 31, ld = G.ld;
-  int64_t A[3], B[3];
-  double wt[3];
+  // sum_s l_e / (A_c d_e) (D_nb - D_c), the own value's weights summed once per cell
+  int64_t B[3];
+  double wt[3], wc = 0.0;
   for (int s = 0; s < 3; ++s) {
     const int e = G.c2e[3 * c + s];
-    A[s] = (int64_t)G.e2c[2 * e] * ld;
-    B[s] = (int64_t)G.e2c[2 * e + 1] * ld;
-    wt[s] = G.div_wa[3 * c + s] * G.inv_de[e];
+    const int ca = G.e2c[2 * e], cb = G.e2c[2 * e + 1];
+    B[s] = (int64_t)(ca == c ? cb : ca) * ld;
+    wt[s] = fabs(G.div_wa[3 * c + s]) * G.inv_de[e];
+    wc += wt[s];
   }
   for (int k = lane; k < G.N; k += 32)
-    L[c * ld + k] = (wt[0] * (D[B[0] + k] - D[A[0] + k]) + wt[1] * (D[B[1] + k] - D[A[1] + k])) +
-                    wt[2] * (D[B[2] + k] - D[A[2] + k]);
+    L[c * ld + k] = fma(wt[2], D[B[2] + k], fma(wt[1], D[B[1] + k], fma(wt[0], D[B[0] + k], -(wc * D[c * ld + k]))));
 }
 
 struct DDArgs {
@@ -348,47 +353,66 @@ __global__ void __launch_bounds__(256, 4) k_dd_edge(Geo64 G, DDArgs a) {
 // ---------------------------------------------------------------- column solve
 //
 // The vertically implicit update of every column in three launches:
-//   k_col_rows   one warp per cell, lanes over levels: everything that is parallel
+//   k_col_rows_*  one warp per cell, lanes over levels: everything that is parallel
 //                over the levels (half-level interpolants, horizontal divergences,
 //                explicit predictors, the linearised state equation, the w predictor
 //                and, in the predictor, the tridiagonal row of every interior half
-//                level, which depends on S^n only and serves both stages). Rows go out
-//                level-major for the solve; the operands of the final update stay in
-//                the cell's own rows.
+//                level). Rows go out level-major for the solve; the operands of the
+//                final update stay in the cell's own rows.
 //   k_col_thomas one thread per column: the Thomas recurrence on level-major rows
 //                (coalesced across the warp; the corrector substitutes with the
-//                predictor's factors), Rayleigh damping; the solution w goes to ws.
+//                predictor's factors), Rayleigh damping; the solution w overwrites
+//                the right-hand side.
 //   k_col_update one warp per cell, lanes over levels: the implicit parts of rho,
 //                Theta and pi, theta_v = Theta / rho, the step-mean vertical mass flux.
 // Only the recurrence is sequential in the level; keeping it apart lets the rest run
 // with coalesced, level-contiguous loads instead of one thread walking a column.
+//
+// The FP64 pipe bounds all three, so whatever depends on S^n only is formed by the predictor
+// and handed to the corrector in buffers that are dead meanwhile: the matrix factors, gamma,
+// the half-level interpolants rho_ic and M, a = dtau beta cpd theta_ic / dzh (in the column's
+// former solution buffer), the w predictor without the stages' advection, plus half the
+// predictor's (in A_w's buffer), and on flat levels the parts of rho and Theta without the
+// horizontal divergences and the same part of Exner's increment. The first two overwrite S^n's
+// rho and theta_v, which nothing else reads until the corrector writes S^{n+1} there: the
+// stencils of the corrector read S*. Exner is carried as its increment delta on S^n's: the
+// pressure term of the row, -a (pi*_{h-1} - pi*_h), splits into S^n's part, which joins the
+// hydrostatic residual of the w predictor (one difference of neighbouring Exner values, exact),
+// and -a (delta_{h-1} - delta_h), which is small; the roundings of pi* no longer enter w.
+// Corrector rows: 18 FP64 instructions per cell-level as written, 35 when it formed them again
+// from S^n. R2B6/90: the column 3.35 ms per launch (mean of the stages), was 3.93.
 struct ColArgs {
-  const double *rho, *thv, *ex, *w;        // S^n [c][ld]
+  // S^n [c][ld]; on flat levels the predictor leaves the explicit parts of rho and Theta
+  // without the horizontal divergences in rho and thv, Exner's increment in d0
+  double *rho, *thv, *d0;
+  const double *ex, *w;
   const double* w_stage;                   // w of the stage state (vertical part of A_w)
-  const double *F, *G, *a_e;               // edge fluxes and w-advection edge terms
-  double* Aw0;                             // stored (predictor) or read (corrector)
-  double *lo, *di, *up, *rh;               // tridiagonal rows, level-major [h][Nc], h = 1..N-1
-  double* ws;                              // the damped solution w^{n+1}, level-major [h][Nc]
-  double *rx, *tx, *px, *gm;               // rho*, Theta*, pi* (explicit parts), gamma: [c][ld]
-  double* gc;                              // (Rd/cvd) pi / Theta of S^n: [c][ld]
+  const double *F, *G, *a_e;               // edge fluxes and d_e times the w-advection edge terms
+  double* ba;                              // w^n - dtau (cpd theta_ic dpi/dz + g) + (dtau/2) A_w0: [c][ld]
+  double* aa;                              // dtau beta cpd theta_ic / dzh: [c][ld]
+  double *lo, *di, *up, *rh;               // tridiagonal rows, level-major [h][Nc], h = 1..N-1; rh becomes w^{n+1}
+  double *rx, *tx, *dx, *gm;               // rho*, Theta*, pi* - pi (explicit parts), gamma: [c][ld]
+  double* gc;                              // (dtau/2) (Rd/cvd) pi / Theta of S^n: [c][ld]
   double *ri, *mm;                         // half-level rho and rho theta_v of S^n: [c][ld]
   double *rho_o, *thv_o, *ex_o, *w_o;      // S* or S^{n+1} (may alias S^n)
   double* wflx;
   unsigned* status;
   double dtau, inv_nsub;
-  double hdtau;                            // dtau / 2 (set on the host: a kernel would recompute it per use)
+  double hdtau, hrc, inv_dtau2;            // dtau / 2, (dtau / 2) Rd/cvd and 2 / dtau (set on the host)
   double b_new, b_old;                     // beta / nsub, (1 - beta) / nsub
-  int corrector;
+  int hdamp;                               // half levels h < hdamp lie in the Rayleigh layer
 };
 
 // windows of 31 levels: lane l holds full level k = base + l and the half level above
-// it (h = k); lane 31 only supplies the half level below lane 30's full level.
+// it (h = k); lane 31 only supplies the half level below lane 30's full level. The level above
+// comes from the neighbouring lane (lane 30's is carried to the next window), never from
+// memory, where this kernel has overwritten it.
 // TOPO (terrain-following levels): each cell's own spacings and interpolation weights,
 // thickness-weighted horizontal fluxes (already carrying dz_e) divided by the cell's dz,
 // the explicit vertical fluxes with the contravariant (1 - beta) w - wcc, and the
-// vertical advection of w with w - wcc.
+// vertical advection of w with w - wcc; S^n stays, since those fluxes change with the stage.
 template <bool TOPO>
-__global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
+__global__ void __launch_bounds__(256, 4) k_col_rows_pred(Geo64 G, ColArgs a) {
   const int64_t c = warp_entity();
   if (c >= G.nc) return;
   const int lane = threadIdx.x & 31, ld = G.ld, N = G.N;
@@ -399,17 +423,24 @@ __global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
   for (int s = 0; s < 3; ++s) {
     E[s] = (int64_t)G.c2e[3 * c + s] * ld;
     dw[s] = G.div_wa_h[3 * c + s];         // the edge fluxes are 2 rho_e vn and 4 rho_e vn theta_e
-    kw[s] = G.kin_w[3 * c + s];
+    kw[s] = G.adv_w[3 * c + s];
   }
-  const double dtau = a.dtau, hdtau = a.hdtau, rcv = kRd / kCvd;
-  double gam_c = 0.0, px_c = 0.0, M_c = 0.0;          // carried: full / half level base - 1
+  const double dtau = a.dtau, hdtau = a.hdtau;
+  double gam_c = 0.0, dx_c = 0.0, M_c = 0.0;          // carried: full / half level base - 1
+  double rho_c = 0.0, thv_c = 0.0, ex_c = 0.0;
   for (int base = 0; base <= N; base += 31) {
     const int k = base + lane;
     const bool hv = k <= N;                            // half level k exists
     const bool kv = lane < 31 && k < N;                // full level k owned here
-    double rho = 0.0, thv = 0.0, ex = 0.0, rho_m = 0.0, thv_m = 0.0, ex_m = 0.0;
+    double rho = 0.0, thv = 0.0, ex = 0.0;
     if (k < N) { rho = a.rho[o + k]; thv = a.thv[o + k]; ex = a.ex[o + k]; }
-    if (k >= 1 && k <= N) { rho_m = a.rho[o + k - 1]; thv_m = a.thv[o + k - 1]; ex_m = a.ex[o + k - 1]; }
+    double rho_m = __shfl_up_sync(0xffffffffu, rho, 1);
+    double thv_m = __shfl_up_sync(0xffffffffu, thv, 1);
+    double ex_m = __shfl_up_sync(0xffffffffu, ex, 1);
+    if (lane == 0) { rho_m = rho_c; thv_m = thv_c; ex_m = ex_c; }
+    rho_c = __shfl_sync(0xffffffffu, rho, 30);
+    thv_c = __shfl_sync(0xffffffffu, thv, 30);
+    ex_c = __shfl_sync(0xffffffffu, ex, 30);
     // half-level interpolants of S^n: rho_ic and M = rho_ic theta_ic
     double ri = 0.0, ti = 0.0;
     if (k == 0) { ri = rho; ti = thv; }
@@ -428,13 +459,11 @@ __global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
     const double M = ri * ti;
     const double wk = hv ? a.w[o + k] : 0.0;
     // TOPO: explicit part of the contravariant velocity at interior half levels
-    const double ve = (TOPO && k >= 1 && k < N) ? (1.0 - kBeta) * wk - G.t_wcc[o + k] : 0.0;
+    const double ve = (TOPO && k >= 1 && k < N) ? (1.0 - kBeta) * wk - G.t_wcc[o + k] : wk;
     const double ri1 = __shfl_down_sync(0xffffffffu, ri, 1);      // half level k + 1
     const double M1 = __shfl_down_sync(0xffffffffu, M, 1);
-    const double w1 = __shfl_down_sync(0xffffffffu, wk, 1);
-    double ve1 = 0.0;
-    if constexpr (TOPO) ve1 = __shfl_down_sync(0xffffffffu, ve, 1);
-    double gam = 0.0, px = 0.0;
+    const double ve1 = __shfl_down_sync(0xffffffffu, (TOPO && (k < 1 || k >= N)) ? 0.0 : ve, 1);
+    double gam = 0.0, dx = 0.0;
     if (kv) {
       // explicit predictors at full level k
       // Dr: the mass-flux divergence; Dt2: twice the heat-flux divergence
@@ -442,78 +471,137 @@ __global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
       for (int s = 0; s < 3; ++s) Dr += dw[s] * a.F[E[s] + k];
       for (int s = 0; s < 3; ++s) Dt2 += dw[s] * a.G[E[s] + k];
       const double Th = rho * thv;
+      const double gd = (a.hrc * ex) * recip64(Th);   // (dtau/2) times the state-equation factor
+      a.gc[o + k] = gd;
       double rx, tx;
       if constexpr (TOPO) {
-        const double idz = G.t_inv_dz_c[o + k];
-        rx = rho - (dtau * ((Dr + ri * ve) - ri1 * ve1)) * idz;
-        tx = Th - (dtau * ((0.5 * Dt2 + M * ve) - M1 * ve1)) * idz;
+        const double v0 = k >= 1 ? ve : 0.0;
+        const double idz = G.t_inv_dz_c[o + k], dti = dtau * idz;
+        rx = rho - dti * ((Dr + ri * v0) - ri1 * ve1);
+        const double dT = dti * ((0.5 * Dt2 + M * v0) - M1 * ve1);
+        tx = Th - dT;
+        dx = -(gd * a.inv_dtau2) * dT;
+        gam = gd * ((2.0 * kBeta) * idz);
       } else {
         const double dt1 = cc[C_DT1BDZ * ld + k];
-        rx = (rho - dtau * Dr) - dt1 * (ri * wk - ri1 * w1);
-        tx = (Th - hdtau * Dt2) - dt1 * (M * wk - M1 * w1);
+        const double Q = M * wk - M1 * ve1;
+        gam = gd * cc[C_2BDZ * ld + k];
+        const double r0 = rho - dt1 * (ri * wk - ri1 * ve1), t0 = Th - dt1 * Q;
+        const double d0 = ((kBeta - 1.0) / kBeta * gam) * Q;
+        rx = r0 - dtau * Dr;
+        tx = t0 - hdtau * Dt2;
+        dx = d0 - gd * Dt2;
+        a.rho[o + k] = r0;
+        a.thv[o + k] = t0;
+        a.d0[o + k] = d0;
       }
-      // the state-equation factor of S^n: formed by the predictor, read back by the corrector
-      double g;
-      if (!a.corrector) {
-        g = (rcv * ex) * recip64(Th);
-        a.gc[o + k] = g;
-      } else {
-        g = a.gc[o + k];
-      }
-      px = ex + g * (tx - Th);
       a.rx[o + k] = rx;
       a.tx[o + k] = tx;
-      a.px[o + k] = px;
-      if (!a.corrector) {
-        if constexpr (TOPO) gam = g * (dtau * kBeta * G.t_inv_dz_c[o + k]);
-        else gam = g * cc[C_DTBDZ * ld + k];
-        a.gm[o + k] = gam;
-      }
+      a.dx[o + k] = dx;
+      a.gm[o + k] = gam;
     }
-    if (hv && lane < 31 && !a.corrector) {
+    if (hv && lane < 31) {
       a.ri[o + k] = ri;
       a.mm[o + k] = M;
     }
     // full level and half level above: from the lane above, or carried for lane 0
     double gam_m = __shfl_up_sync(0xffffffffu, gam, 1);
-    double px_m = __shfl_up_sync(0xffffffffu, px, 1);
+    double dx_m = __shfl_up_sync(0xffffffffu, dx, 1);
     double M_m = __shfl_up_sync(0xffffffffu, M, 1);
-    if (lane == 0) { gam_m = gam_c; px_m = px_c; M_m = M_c; }
+    if (lane == 0) { gam_m = gam_c; dx_m = dx_c; M_m = M_c; }
     if (kv && k >= 1) {
       // row of interior half level h = k: w predictor and the implicit coupling
       const int h = k;
       double hadv = 0.0;
       for (int s = 0; s < 3; ++s) hadv += kw[s] * a.a_e[E[s] + h];
-      const double ws = a.w_stage[o + h];
-      double Aw;
-      if constexpr (TOPO)
-        Aw = -hadv - G.t_wcon[o + h] * (a.w_stage[o + h - 1] - a.w_stage[o + h + 1]) * (0.5 * G.t_inv_dzh_c[o + h]);
-      else
-        Aw = -hadv - ws * (a.w_stage[o + h - 1] - a.w_stage[o + h + 1]) * G.inv_dz2[h];
-      if (a.corrector) Aw = 0.5 * (a.Aw0[o + h] + Aw);
-      else a.Aw0[o + h] = Aw;
-      const double th_ic = ti;
-      double w_x, aa;
+      const double* ws = a.w_stage + o + h;
+      double Aw, B, aa;
       if constexpr (TOPO) {
         const double idzh = G.t_inv_dzh_c[o + h];
-        w_x = wk + dtau * ((Aw - ((1.0 - kBeta) * kCpd * idzh) * th_ic * (ex_m - ex)) - kGrav);
-        aa = (dtau * kBeta * kCpd * idzh) * th_ic;
+        Aw = -hadv - G.t_wcon[o + h] * (ws[-1] - ws[1]) * (0.5 * idzh);
+        B = wk + dtau * (-((kCpd * idzh) * ti) * (ex_m - ex) - kGrav);
+        aa = (dtau * kBeta * kCpd * idzh) * ti;
       } else {
-        w_x = wk + dtau * ((Aw - cc[C_CX * ld + h] * th_ic * (ex_m - ex)) - kGrav);
-        aa = cc[C_CA * ld + h] * th_ic;
+        Aw = -hadv - ws[0] * (ws[-1] - ws[1]) * G.inv_dz2[h];
+        B = wk + dtau * (-(cc[C_CX * ld + h] * ti) * (ex_m - ex) - kGrav);
+        aa = cc[C_CA * ld + h] * ti;
       }
+      a.ba[o + h] = B + hdtau * Aw;
+      a.aa[o + h] = aa;
       const int64_t i = (int64_t)h * nc + c;
-      if (!a.corrector) {
-        const double P = aa * gam_m, Q = aa * gam;
-        a.lo[i] = -P * M_m;
-        a.di[i] = fma(P + Q, M, 1.0);
-        a.up[i] = -Q * M1;
-      }
-      a.rh[i] = w_x - aa * (px_m - px);
+      const double P = aa * gam_m, Q = aa * gam;
+      a.lo[i] = -P * M_m;
+      a.di[i] = fma(P + Q, M, 1.0);
+      a.up[i] = -Q * M1;
+      a.rh[i] = (B + dtau * Aw) - aa * (dx_m - dx);
     }
     gam_c = __shfl_sync(0xffffffffu, gam, 30);
-    px_c = __shfl_sync(0xffffffffu, px, 30);
+    dx_c = __shfl_sync(0xffffffffu, dx, 30);
     M_c = __shfl_sync(0xffffffffu, M, 30);
+  }
+}
+
+// the corrector's right-hand side and explicit parts, from what the predictor left. Flat levels
+// need the level above only: windows of 32 with lane 31's carried.
+template <bool TOPO>
+__global__ void __launch_bounds__(256, 4) k_col_rows_corr(Geo64 G, ColArgs a) {
+  const int64_t c = warp_entity();
+  if (c >= G.nc) return;
+  const int lane = threadIdx.x & 31, ld = G.ld, N = G.N;
+  const int64_t o = c * ld, nc = G.nc;
+  int64_t E[3];
+  double dw[3], kw[3];
+  for (int s = 0; s < 3; ++s) {
+    E[s] = (int64_t)G.c2e[3 * c + s] * ld;
+    dw[s] = G.div_wa_h[3 * c + s];
+    kw[s] = G.adv_w[3 * c + s];
+  }
+  const double dtau = a.dtau, hdtau = a.hdtau;
+  constexpr int W = TOPO ? 31 : 32;
+  double dx_c = 0.0;                                   // carried: full level base - 1
+  for (int base = 0; base < N; base += W) {
+    const int k = base + lane;
+    const bool kv = lane < W && k < N;
+    double ve = 0.0, ve1 = 0.0;
+    if constexpr (TOPO) {
+      if (k >= 1 && k < N) ve = (1.0 - kBeta) * a.w[o + k] - G.t_wcc[o + k];
+      ve1 = __shfl_down_sync(0xffffffffu, ve, 1);
+    }
+    double dx = 0.0;
+    if (kv) {
+      double Dr = 0.0, Dt2 = 0.0;
+      for (int s = 0; s < 3; ++s) Dr += dw[s] * a.F[E[s] + k];
+      for (int s = 0; s < 3; ++s) Dt2 += dw[s] * a.G[E[s] + k];
+      const double gd = a.gc[o + k];
+      double rx, tx;
+      if constexpr (TOPO) {
+        const double rho = a.rho[o + k], Th = rho * a.thv[o + k], dti = dtau * G.t_inv_dz_c[o + k];
+        rx = rho - dti * ((Dr + a.ri[o + k] * ve) - a.ri[o + k + 1] * ve1);
+        const double dT = dti * ((0.5 * Dt2 + a.mm[o + k] * ve) - a.mm[o + k + 1] * ve1);
+        tx = Th - dT;
+        dx = -(gd * a.inv_dtau2) * dT;
+      } else {
+        rx = a.rho[o + k] - dtau * Dr;
+        tx = a.thv[o + k] - hdtau * Dt2;
+        dx = a.d0[o + k] - gd * Dt2;
+      }
+      a.rx[o + k] = rx;
+      a.tx[o + k] = tx;
+      a.dx[o + k] = dx;
+    }
+    double dx_m = __shfl_up_sync(0xffffffffu, dx, 1);
+    if (lane == 0) dx_m = dx_c;
+    dx_c = __shfl_sync(0xffffffffu, dx, W - 1);
+    if (kv && k >= 1) {
+      const int h = k;
+      double hadv = 0.0;
+      for (int s = 0; s < 3; ++s) hadv += kw[s] * a.a_e[E[s] + h];
+      const double* ws = a.w_stage + o + h;
+      double Aw;
+      if constexpr (TOPO) Aw = -hadv - G.t_wcon[o + h] * (ws[-1] - ws[1]) * (0.5 * G.t_inv_dzh_c[o + h]);
+      else Aw = -hadv - ws[0] * (ws[-1] - ws[1]) * G.inv_dz2[h];
+      a.rh[(int64_t)h * nc + c] = (a.ba[o + h] + hdtau * Aw) - a.aa[o + h] * (dx_m - dx);
+    }
   }
 }
 
@@ -522,8 +610,8 @@ __global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
 // S^n only (rho_ic, theta_ic and the state-equation factor of the substep's start), so it is
 // the same in both stages: the predictor factors it, keeping the sub-diagonal, storing
 // 1 / pivot over the diagonal and up / pivot over the super-diagonal, and the corrector only
-// substitutes its own right-hand side (the same operations on the same values as a second
-// factorisation, so the results are unchanged). The damped solution goes to ws.
+// substitutes its own right-hand side. The damped solution goes over the right-hand side.
+template <bool CORR>
 __global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= G.nc) return;
@@ -535,9 +623,8 @@ __global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
   double* __restrict__ di = a.di;
   double* __restrict__ up = a.up;
   double* __restrict__ rh = a.rh;
-  double* __restrict__ ws = a.ws;
   double dp = 0.0;
-  if (!a.corrector) {
+  if (!CORR) {
     double cp = 0.0;
     double l = lo[nc + c], d = di[nc + c], u = up[nc + c], r = rh[nc + c];
     for (int h = 1; h < N; ++h) {
@@ -570,17 +657,17 @@ __global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
   }
   // back substitution
   double x = dp;
-  ws[(int64_t)(N - 1) * nc + c] = x * cc[C_DAMP * ld + N - 1];
+  if (N - 1 < a.hdamp) rh[(int64_t)(N - 1) * nc + c] = x * cc[C_DAMP * ld + N - 1];
   for (int h = N - 2; h >= 1; --h) {
     const int64_t i = (int64_t)h * nc + c;
     x = rh[i] - up[i] * x;
-    ws[i] = x * cc[C_DAMP * ld + h];
+    rh[i] = h < a.hdamp ? x * cc[C_DAMP * ld + h] : x;
   }
 }
 
 // TOPO: each cell's dz, the contravariant step-mean vertical flux, and the ground w of
 // the stage (its wcc, so that w - wcc = 0 there)
-template <bool TOPO>
+template <bool TOPO, bool CORR>
 __global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
   const int64_t c = warp_entity();
   if (c >= G.nc) return;
@@ -591,7 +678,7 @@ __global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
   for (int base = 0; base < N; base += 31) {
     const int k = base + lane;
     // w^{n+1} (damped) at half level k; zero at the top and the bottom
-    const double wn = (k >= 1 && k < N) ? a.ws[(int64_t)k * nc + c] : 0.0;
+    const double wn = (k >= 1 && k < N) ? a.rh[(int64_t)k * nc + c] : 0.0;
     const double ri = k <= N ? a.ri[o + k] : 0.0;
     const double M = k <= N ? a.mm[o + k] : 0.0;
     const double wn1 = __shfl_down_sync(0xffffffffu, wn, 1);
@@ -602,10 +689,10 @@ __global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
       const double r = ri * wn - ri1 * wn1;
       const double dtb = TOPO ? a.dtau * kBeta * G.t_inv_dz_c[o + k] : cc[C_DTBDZ * ld + k];
       const double Th_n = a.tx[o + k] - dtb * q;
-      const double ex_n = a.px[o + k] - a.gm[o + k] * q;
+      const double ex_n = a.ex[o + k] + (a.dx[o + k] - a.gm[o + k] * q);
       const double rho_n = a.rx[o + k] - dtb * r;
       const double thv_n = Th_n * recip64(rho_n);
-      if (a.corrector) {
+      if (CORR) {
         // (beta wn + (1 - beta) wold - wcc) / nsub with the weights divided on the host
         const double wold = a.w[o + k];
         double wc = fma(a.b_new, wn, a.b_old * wold);
@@ -667,10 +754,6 @@ __global__ void __launch_bounds__(256) k_diff_div(Geo64 G, const double* __restr
   }
 }
 
-__device__ inline double dot3(double ax, double ay, double az, const double* b) {
-  return (ax * b[0] + ay * b[1]) + az * b[2];
-}
-
 // fourth-order background diffusion (option): L1 = L(vn) at edges, then the divergence
 // and curl of L1 for the second Laplacian in k_diff_edge
 __global__ void __launch_bounds__(256, 4) k_bd_lap(Geo64 G, const double* __restrict__ zeta,
@@ -707,11 +790,11 @@ struct BDArgs {
   double scale;                            // c Abar^2
 };
 
-__global__ void __launch_bounds__(256, 4) k_diff_edge(Geo64 G, double* __restrict__ vn, const double* __restrict__ ux,
+__global__ void __launch_bounds__(256, 3) k_diff_edge(Geo64 G, double* __restrict__ vn, const double* __restrict__ ux,
                                                    const double* __restrict__ uy, const double* __restrict__ uz,
                                                    const double* __restrict__ zeta, const double* __restrict__ divc,
-                                                   const double* __restrict__ thv, double* __restrict__ Kh_out,
-                                                   double* __restrict__ thflx, double dt, BDArgs bd) {
+                                                   const double* __restrict__ thv, double* __restrict__ thflx,
+                                                   double dt, BDArgs bd) {
   const int64_t e = warp_entity();
   if (e >= G.ne) return;
   const int lane = threadIdx.x & 31, ld = G.ld;
@@ -719,27 +802,37 @@ __global__ void __launch_bounds__(256, 4) k_diff_edge(Geo64 G, double* __restric
   for (int j = 0; j < 4; ++j) Q[j] = (int64_t)G.e2q[4 * e + j] * ld;
   const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
   const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
-  const double* n = G.n_e + 3 * e;
-  const double* t = G.t_e + 3 * e;
-  const double le = G.l_e[e], de = G.d_e[e], i34 = G.inv_L34[e], ile = G.inv_le[e], ide = G.inv_de[e];
-  const double cs2ld = (kCsSmag * kCsSmag) * (le * de);
+  const double ile = G.inv_le[e], ide = G.inv_de[e], i34 = G.inv_L34[e];
+  // the normal and the tangent scaled by 1/L34 and 1/l_e once per edge, and the factors of the
+  // two products that K_h enters
+  double n34[3], t34[3], n12[3], t12[3];
+  for (int j = 0; j < 3; ++j) {
+    const double n = G.n_e[3 * e + j], t = G.t_e[3 * e + j];
+    n34[j] = n * i34;
+    t34[j] = t * i34;
+    n12[j] = n * ile;
+    t12[j] = t * ile;
+  }
+  const double cs2ld = (kCsSmag * kCsSmag) * (G.l_e[e] * G.d_e[e]);
+  const double dtk = dt * cs2ld, fk = (G.l_e[e] * ide) * cs2ld;
   for (int k = lane; k < G.N; k += 32) {
     const double d34x = ux[Q[3] + k] - ux[Q[2] + k], d34y = uy[Q[3] + k] - uy[Q[2] + k],
                  d34z = uz[Q[3] + k] - uz[Q[2] + k];
     const double d12x = ux[Q[1] + k] - ux[Q[0] + k], d12y = uy[Q[1] + k] - uy[Q[0] + k],
                  d12z = uz[Q[1] + k] - uz[Q[0] + k];
-    const double DT = dot3(d34x, d34y, d34z, n) * i34 - dot3(d12x, d12y, d12z, t) * ile;
-    const double DS = dot3(d34x, d34y, d34z, t) * i34 + dot3(d12x, d12y, d12z, n) * ile;
-    const double Kh = cs2ld * sqrt(DT * DT + DS * DS);
+    const double DT = fma(d34z, n34[2], fma(d34y, n34[1], d34x * n34[0])) -
+                      fma(d12z, t12[2], fma(d12y, t12[1], d12x * t12[0]));
+    const double DS = fma(d12z, n12[2], fma(d12y, n12[1], fma(d12x, n12[0],
+                      fma(d34z, t34[2], fma(d34y, t34[1], d34x * t34[0])))));
+    const double D = sqrt64(fma(DS, DS, DT * DT));
     const double lap = (divc[c2 + k] - divc[c1 + k]) * ide - (zeta[v2 + k] - zeta[v1 + k]) * ile;
-    double vnew = vn[e * ld + k] + dt * Kh * lap;
+    double vnew = fma(dtk * D, lap, vn[e * ld + k]);
     if (bd.D1) {
       const double lap2 = (bd.D1[c2 + k] - bd.D1[c1 + k]) * ide - (bd.zeta1[v2 + k] - bd.zeta1[v1 + k]) * ile;
       vnew -= bd.scale * lap2;
     }
     vn[e * ld + k] = vnew;
-    Kh_out[e * ld + k] = Kh;
-    thflx[e * ld + k] = (le * Kh) * (thv[c2 + k] - thv[c1 + k]) * ide;
+    thflx[e * ld + k] = (fk * D) * (thv[c2 + k] - thv[c1 + k]);
   }
 }
 
@@ -777,19 +870,24 @@ Geo64 make_geo(const icon_grid* grid, const double* cc) {
   G.inv_L34 = g.inv_L34; G.n_e = g.n_e; G.t_e = g.t_e; G.s_ce = g.s_ce;
   G.wu = v.d_wu; G.wl = v.d_wl; G.inv_dz = v.d_inv_dz; G.inv_dz2 = v.d_inv_dz2; G.qinv_dz = v.d_qinv_dz;
   G.cc = cc;
-  G.kin_w_h = G.div_wa_h = nullptr;
+  G.kin_w_h = G.div_wa_h = G.adv_w = nullptr;
   G.t_sn = G.t_bf = G.t_wu_e = G.t_qinv_dz_e = G.t_dz_e = nullptr;
   G.t_wu_c = G.t_inv_dz_c = G.t_inv_dzh_c = G.t_wcc = G.t_wcon = G.t_ep = G.t_hdpdz = nullptr;
   return G;
 }
 
-void launch_column(const Geo64& G, const ColArgs& a, bool topo, cudaStream_t st) {
-  const unsigned nbc = blocks_for(G.nc, kWarpsPerBlock);
-  if (topo) k_col_rows<true><<<nbc, 256, 0, st>>>(G, a);
-  else k_col_rows<false><<<nbc, 256, 0, st>>>(G, a);
-  k_col_thomas<<<blocks_for(G.nc, 128), 128, 0, st>>>(G, a);
-  if (topo) k_col_update<true><<<nbc, 256, 0, st>>>(G, a);
-  else k_col_update<false><<<nbc, 256, 0, st>>>(G, a);
+template <bool TOPO>
+void launch_column(const Geo64& G, const ColArgs& a, bool corr, cudaStream_t st) {
+  const unsigned nbc = blocks_for(G.nc, kWarpsPerBlock), nbt = blocks_for(G.nc, 128);
+  if (corr) {
+    k_col_rows_corr<TOPO><<<nbc, 256, 0, st>>>(G, a);
+    k_col_thomas<true><<<nbt, 128, 0, st>>>(G, a);
+    k_col_update<TOPO, true><<<nbc, 256, 0, st>>>(G, a);
+  } else {
+    k_col_rows_pred<TOPO><<<nbc, 256, 0, st>>>(G, a);
+    k_col_thomas<false><<<nbt, 128, 0, st>>>(G, a);
+    k_col_update<TOPO, false><<<nbc, 256, 0, st>>>(G, a);
+  }
 }
 
 }  // namespace
@@ -801,6 +899,7 @@ Geo64 state_geo(const icon_state* st) {
   Geo64 G = make_geo(st->grid, s.colconst);
   G.kin_w_h = s.kin_w_h;
   G.div_wa_h = s.div_wa_h;
+  G.adv_w = s.adv_w;
   const TopoDev& T = s.topo;
   if (T.on) {
     G.t_sn = T.sn; G.t_bf = T.bf; G.t_wu_e = T.wu_e; G.t_qinv_dz_e = T.qinv_dz_e; G.t_dz_e = T.dz_e;
@@ -887,9 +986,9 @@ void fp64_step_stage(icon_state* st, double dt, int nsub, bool corr, cudaStream_
   ca.rho = s.rho; ca.thv = s.thv; ca.ex = s.ex; ca.w = s.w;
   ca.w_stage = w_st;
   ca.F = s.F; ca.G = s.G; ca.a_e = s.a_e;
-  ca.Aw0 = s.Aw0;
-  ca.lo = s.col_lo; ca.di = s.col_di; ca.up = s.col_up; ca.rh = s.col_rh; ca.ws = s.col_ws;
-  ca.rx = s.col_rx; ca.tx = s.col_tx; ca.px = s.col_px; ca.gm = s.col_gm;
+  ca.ba = s.Aw0; ca.aa = s.col_ws;
+  ca.lo = s.col_lo; ca.di = s.col_di; ca.up = s.col_up; ca.rh = s.col_rh;
+  ca.rx = s.col_rx; ca.tx = s.col_tx; ca.dx = s.col_px; ca.gm = s.col_gm; ca.d0 = s.col_d0;
   ca.ri = s.col_ri; ca.mm = s.col_mm; ca.gc = s.col_gc;
   ca.rho_o = corr ? s.rho : s.rho_s;
   ca.thv_o = corr ? s.thv : s.thv_s;
@@ -897,12 +996,17 @@ void fp64_step_stage(icon_state* st, double dt, int nsub, bool corr, cudaStream_
   ca.w_o = corr ? s.w : s.w_s;
   ca.wflx = s.wflx;
   ca.status = s.status;
-  ca.dtau = dtau; ca.inv_nsub = 1.0 / nsub; ca.corrector = corr;
-  ca.hdtau = 0.5 * dtau;
+  ca.dtau = dtau; ca.hdtau = 0.5 * dtau; ca.inv_nsub = 1.0 / nsub;
+  ca.hrc = 0.5 * dtau * (kRd / kCvd); ca.inv_dtau2 = 2.0 / dtau;
   ca.b_new = kBeta / nsub;
   ca.b_old = (1.0 - kBeta) / nsub;
+  ca.hdamp = 0;
+  const std::vector<double>& ray = st->grid->vert.rayleigh;
+  for (int h = 0; h <= G.N; ++h)
+    if (ray[h] > 0.0) ca.hdamp = h + 1;
   prof_begin(stream, K_COLUMN);
-  launch_column(G, ca, topo, stream);
+  if (topo) launch_column<true>(G, ca, corr, stream);
+  else launch_column<false>(G, ca, corr, stream);
   prof_end(stream);
 }
 
@@ -930,7 +1034,7 @@ void fp64_step_diffusion(icon_state* st, double dt, cudaStream_t stream) {
     bd.D1 = s.col_lo; bd.zeta1 = s.col_di; bd.scale = st->diff4 * abar * abar;
   }
   prof_begin(stream, K_DIFF_EDGE);
-  k_diff_edge<<<nbe, 256, 0, stream>>>(G, s.vn, s.uvx, s.uvy, s.uvz, s.zeta, s.divc, s.thv, s.Kh, s.thflx, dt, bd);
+  k_diff_edge<<<nbe, 256, 0, stream>>>(G, s.vn, s.uvx, s.uvy, s.uvz, s.zeta, s.divc, s.thv, s.thflx, dt, bd);
   prof_end(stream);
   prof_begin(stream, K_DIFF_THETA);
   k_diff_theta<<<nbc, 256, 0, stream>>>(G, s.thflx, s.thv, s.ex, dt);

@@ -173,7 +173,8 @@ struct StateDev {
   // half the cell weights kappa_ce and s_ce l_e / A_c ([Nc][3]): the FP64 step stores
   // 2 K_e, 2 rho_e vn and 4 rho_e vn theta_e at edges and folds the factors in here
   double *kin_w_h = nullptr, *div_wa_h = nullptr;
-  double *uvx = nullptr, *uvy = nullptr, *uvz = nullptr, *divc = nullptr, *Kh = nullptr, *thflx = nullptr;
+  double* adv_w = nullptr;             // kappa_ce / d_e ([Nc][3]): the FP64 step stores d_e a_e at edges
+  double *uvx = nullptr, *uvy = nullptr, *uvz = nullptr, *divc = nullptr, *thflx = nullptr;
   // mixed-mode scratch and shadows
   float *zeta32 = nullptr, *wv32 = nullptr, *vt32 = nullptr, *Ke32 = nullptr, *Kc32 = nullptr,
         *ae32 = nullptr, *F32 = nullptr, *G32 = nullptr;
@@ -188,6 +189,7 @@ struct StateDev {
   double *col_lo = nullptr, *col_di = nullptr, *col_up = nullptr, *col_rh = nullptr;
   double *col_rx = nullptr, *col_tx = nullptr, *col_px = nullptr, *col_gm = nullptr;
   double *col_ri = nullptr, *col_mm = nullptr, *col_ws = nullptr, *col_gc = nullptr;
+  double* col_d0 = nullptr;            // flat levels only
   double* colconst = nullptr;
   // tracers (mixing ratios, FP64 [t][Nc][ld]) and their transport scratch
   int ntr = 0;

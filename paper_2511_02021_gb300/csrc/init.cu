@@ -259,6 +259,13 @@ __global__ void k_mixed_cells(int64_t nc, int64_t c0, int64_t n, int N, int ld, 
   }
 }
 
+// kappa_ce / d_e per cell and edge slot
+__global__ void k_adv_w(const double* __restrict__ kin_w, const int* __restrict__ c2e,
+                        const double* __restrict__ inv_de, double* __restrict__ out, int64_t n) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) out[i] = kin_w[i] * inv_de[c2e[i]];
+}
+
 __global__ void k_half(const double* __restrict__ a, double* __restrict__ b, int64_t n) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) b[i] = 0.5 * a[i];
@@ -346,6 +353,7 @@ int init_state_device(icon_state* st, uint64_t seed, int case_id, const icon_cas
   if (s.precision == ICON_FP64) {
     k_half<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.kin_w, s.kin_w_h, 3 * g.nc);
     k_half<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.div_wa, s.div_wa_h, 3 * g.nc);
+    k_adv_w<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.kin_w, g.c2e, g.inv_de, s.adv_w, 3 * g.nc);
     const TopoDev& T = s.topo;
     k_init_cells<<<blocks_for(g.nc, 128), 128, 0, stream>>>(cd, 0, g.nc, g.x_c, v.d_z_f, v.d_dzh, v.d_wu, v.d_wl,
                                                             T.on ? T.hs : nullptr, T.bf, T.wu_c, s.rho, s.thv,
