@@ -256,6 +256,7 @@ int alloc_state(icon_state* st, int precision, bool topo) {
     s.a_e = A.get_n<double>(E); s.F = A.get_n<double>(E); s.G = A.get_n<double>(E);
     s.kin_w_h = A.get_n<double>(3 * (size_t)nc); s.div_wa_h = A.get_n<double>(3 * (size_t)nc);
     s.adv_w = A.get_n<double>(3 * (size_t)nc);
+    s.edge_c = A.get_n<double>(4 * (size_t)ne); s.lap_w = A.get_n<double>(4 * (size_t)nc);
     // diffusion scratch reuses substep scratch (they never overlap in time)
     s.thflx = s.Ke; s.divc = s.Kc; s.uvx = s.w_v;
     s.uvy = A.get_n<double>(V); s.uvz = A.get_n<double>(V);

@@ -57,11 +57,16 @@ struct Geo64 {
   const double* cc;                        // per-level constants for the current dtau
   const double *kin_w_h, *div_wa_h;        // half the cell weights (state tables, [Nc][3])
   const double* adv_w;                     // kappa_ce / d_e (state table, [Nc][3]): w advection
+  // what the stencils would otherwise form per warp (a warp serves one entity in three windows of
+  // levels, so an instruction per entity costs as much as a third of one per level): per edge
+  // [Ne][4] 1/d_e, f_e, d_e / (6 l_e), -cpd / (2 d_e); per cell [Nc][4] the damping Laplacian's
+  // weights l_e / (A_c d_e) of the three neighbours and their sum
+  const double4 *edge_c, *lap_w;
   // terrain-following levels (the TOPO kernel variants; see terrain.cu): per-edge normal
-  // slope factor, full-level decay, per-entity tables [entity][ld], and the stage's
+  // slope factor times cpd / 2, full-level decay, per-entity tables [entity][ld], and the stage's
   // contravariant correction, contravariant velocity, Exner perturbation and half its
   // vertical derivative
-  const double *t_sn, *t_bf, *t_wu_e, *t_qinv_dz_e, *t_dz_e;
+  const double *t_hsn, *t_bf, *t_wu_e, *t_qinv_dz_e, *t_dz_e;
   const double *t_wu_c, *t_inv_dz_c, *t_inv_dzh_c, *t_wcc, *t_wcon, *t_ep, *t_hdpdz;
 };
 
@@ -186,7 +191,7 @@ struct EdgeArgs {
 // half levels in windows of 31 (lane l of a window holds half level h = base + l and,
 // for l < 31, full level k = h), each half-level interpolant and cell-pair sum formed
 // once and handed to the lane below with a shuffle, factors of 1/2 folded into
-// exactly-scaled constants, and the per-edge constants cpd / d_e hoisted.
+// exactly-scaled constants, and the per-edge constants read from a table.
 //
 // TOPO (terrain-following levels): per-edge interpolation weights, the contravariant
 // vertical velocity w - wcc (zero at lid and ground) in the vertical advection of vn,
@@ -202,16 +207,14 @@ __global__ void __launch_bounds__(256, 4) k_edge_tend(Geo64 G, EdgeArgs a) {
   const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
   const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
   const int64_t eo = e * ld;
-  const double ide = G.inv_de[e], fe = G.f_e[e];
-  // a_e is stored times d_e (the cells' weights carry 1/d_e); w_v is six times the mean
-  const double rt = (G.inv_le[e] * G.d_e[e]) * (1.0 / 6.0);
-  // the factors 1/2 of theta_e = (t1 + t2)/2 and rho_e = (rho1 + rho2)/2 are folded into
-  // these constants (and the column's divergence weights), exact scalings by powers of two
-  const double hcide = 0.5 * (kCpd * ide);
-  const double hcsne = TOPO ? 0.5 * (kCpd * G.t_sn[e]) : 0.0;
-  // flat levels: the pressure-gradient term enters vn through one multiply-add with
-  // -dtau cpd / (2 d_e), and the advective part through dtau (predictor) or dtau / 2
-  const double ndhcide = -(a.dtau * hcide);
+  // 1/d_e; f_e; d_e / (6 l_e) (a_e is stored times d_e, the cells' weights carry 1/d_e, and w_v is
+  // six times the mean); -cpd / (2 d_e), or -cpd / d_e in the corrector. The factors 1/2 of
+  // theta_e = (t1 + t2)/2 and rho_e = (rho1 + rho2)/2 are in the last one and in the column's
+  // divergence weights, exact scalings by powers of two
+  const double4 ec = G.edge_c[e];
+  const double ide = ec.x, fe = ec.y, rt = ec.z;
+  const double npg = (!TOPO && a.corrector) ? ec.w + ec.w : ec.w;
+  const double hsn = TOPO ? G.t_hsn[e] : 0.0;
   const double hinv_nsub = a.hinv_nsub;
   const double* __restrict__ vn = a.vn + eo;
   const double* __restrict__ vt = a.vt + eo;
@@ -258,20 +261,21 @@ __global__ void __launch_bounds__(256, 4) k_edge_tend(Geo64 G, EdgeArgs a) {
       const double th_s = t1 + t2;                     // 2 theta_e
       double vnew;
       if (TOPO) {
-        const double corr = (hcsne * G.t_bf[k]) * (G.t_hdpdz[c1 + k] + G.t_hdpdz[c2 + k]);
-        const double pg = th_s * fma(G.t_ep[c2 + k] - G.t_ep[c1 + k], hcide, -corr);
+        // X: the pressure gradient over theta_e / 2, downgradient
+        const double X = fma(G.t_ep[c2 + k] - G.t_ep[c1 + k], npg,
+                             (hsn * G.t_bf[k]) * (G.t_hdpdz[c1 + k] + G.t_hdpdz[c2 + k]));
         if (a.corrector) {
-          vnew = fma(dtau, fma(0.5, a.Avn0[eo + k] + A, -pg), a.vn_base[eo + k]);
+          vnew = fma(dtau, fma(0.5, a.Avn0[eo + k] + A, th_s * X), a.vn_base[eo + k]);
         } else {
-          vnew = fma(dtau, A - pg, a.vn_base[eo + k]);
+          vnew = fma(dtau, fma(th_s, X, A), a.vn_base[eo + k]);
           a.Avn0[eo + k] = A;
         }
       } else {
         const double tdx = th_s * (a.ex[c2 + k] - a.ex[c1 + k]);
         if (a.corrector) {
-          vnew = fma(ndhcide, tdx, fma(a.hdtau, a.Avn0[eo + k] + A, a.vn_base[eo + k]));
+          vnew = fma(a.hdtau, fma(npg, tdx, a.Avn0[eo + k] + A), a.vn_base[eo + k]);
         } else {
-          vnew = fma(ndhcide, tdx, fma(dtau, A, a.vn_base[eo + k]));
+          vnew = fma(dtau, fma(npg, tdx, A), a.vn_base[eo + k]);
           a.Avn0[eo + k] = A;
         }
       }
@@ -310,25 +314,23 @@ __global__ void __launch_bounds__(256, 4) k_dd_lap(Geo64 G, const double* __rest
   const int64_t c = warp_entity();
   if (c >= G.nc) return;
   const int lane = threadIdx.x & 31, ld = G.ld;
-  // sum_s l_e / (A_c d_e) (D_nb - D_c), the own value's weights summed once per cell
+  // sum_s l_e / (A_c d_e) (D_nb - D_c), the own value's weights summed
   int64_t B[3];
-  double wt[3], wc = 0.0;
   for (int s = 0; s < 3; ++s) {
     const int e = G.c2e[3 * c + s];
     const int ca = G.e2c[2 * e], cb = G.e2c[2 * e + 1];
     B[s] = (int64_t)(ca == c ? cb : ca) * ld;
-    wt[s] = fabs(G.div_wa[3 * c + s]) * G.inv_de[e];
-    wc += wt[s];
   }
+  const double4 w = G.lap_w[c];
   for (int k = lane; k < G.N; k += 32)
-    L[c * ld + k] = fma(wt[2], D[B[2] + k], fma(wt[1], D[B[1] + k], fma(wt[0], D[B[0] + k], -(wc * D[c * ld + k]))));
+    L[c * ld + k] = fma(w.z, D[B[2] + k], fma(w.y, D[B[1] + k], fma(w.x, D[B[0] + k], -(w.w * D[c * ld + k]))));
 }
 
 struct DDArgs {
   const double *L, *rho, *thv;             // Laplacian of the divergence, stage state S*
   double *vn, *F, *G, *mflx;
   const double* dz_e;                      // layer thickness at edges (terrain-following), or NULL
-  double scale, inv_nsub;                  // c4 Abar^2
+  double scale, hinv_nsub;                 // c4 Abar^2, 1 / (2 nsub)
   int upwind_theta;
 };
 
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(256, 4) k_dd_edge(Geo64 G, DDArgs a) {
     a.F[eo + k] = F;
     const double t1 = a.thv[c1 + k], t2 = a.thv[c2 + k];
     a.G[eo + k] = F * (a.upwind_theta ? (vn >= 0.0 ? t1 + t1 : t2 + t2) : t1 + t2);
-    a.mflx[eo + k] = fma(F, 0.5 * a.inv_nsub, a.mflx[eo + k]);
+    a.mflx[eo + k] = fma(F, a.hinv_nsub, a.mflx[eo + k]);
   }
 }
 
@@ -871,7 +873,8 @@ Geo64 make_geo(const icon_grid* grid, const double* cc) {
   G.wu = v.d_wu; G.wl = v.d_wl; G.inv_dz = v.d_inv_dz; G.inv_dz2 = v.d_inv_dz2; G.qinv_dz = v.d_qinv_dz;
   G.cc = cc;
   G.kin_w_h = G.div_wa_h = G.adv_w = nullptr;
-  G.t_sn = G.t_bf = G.t_wu_e = G.t_qinv_dz_e = G.t_dz_e = nullptr;
+  G.edge_c = G.lap_w = nullptr;
+  G.t_hsn = G.t_bf = G.t_wu_e = G.t_qinv_dz_e = G.t_dz_e = nullptr;
   G.t_wu_c = G.t_inv_dz_c = G.t_inv_dzh_c = G.t_wcc = G.t_wcon = G.t_ep = G.t_hdpdz = nullptr;
   return G;
 }
@@ -900,9 +903,11 @@ Geo64 state_geo(const icon_state* st) {
   G.kin_w_h = s.kin_w_h;
   G.div_wa_h = s.div_wa_h;
   G.adv_w = s.adv_w;
+  G.edge_c = reinterpret_cast<const double4*>(s.edge_c);
+  G.lap_w = reinterpret_cast<const double4*>(s.lap_w);
   const TopoDev& T = s.topo;
   if (T.on) {
-    G.t_sn = T.sn; G.t_bf = T.bf; G.t_wu_e = T.wu_e; G.t_qinv_dz_e = T.qinv_dz_e; G.t_dz_e = T.dz_e;
+    G.t_hsn = T.hsn; G.t_bf = T.bf; G.t_wu_e = T.wu_e; G.t_qinv_dz_e = T.qinv_dz_e; G.t_dz_e = T.dz_e;
     G.t_wu_c = T.wu_c; G.t_inv_dz_c = T.inv_dz_c; G.t_inv_dzh_c = T.inv_dzh_c;
     G.t_wcc = T.wcc; G.t_wcon = T.wcon; G.t_ep = T.ep; G.t_hdpdz = T.hdpdz;
   }
@@ -974,7 +979,7 @@ void fp64_step_stage(icon_state* st, double dt, int nsub, bool corr, cudaStream_
     da.L = s.col_rx; da.rho = rho_st; da.thv = thv_st;
     da.vn = s.vn; da.F = s.F; da.G = s.G; da.mflx = s.mflx;
     da.dz_e = topo ? T.dz_e : nullptr;
-    da.scale = st->divdamp4 * abar * abar; da.inv_nsub = 1.0 / nsub;
+    da.scale = st->divdamp4 * abar * abar; da.hinv_nsub = 0.5 / nsub;
     da.upwind_theta = st->upwind_theta ? 1 : 0;
     prof_begin(stream, K_DIVDAMP);
     k_dd_div<<<nbc, 256, 0, stream>>>(G, s.vn, s.Kc);

@@ -133,6 +133,8 @@ struct TopoDev {
   double* hs = nullptr;               // [Nc] surface height
   double *b = nullptr, *bf = nullptr; // [ld] decay at half and full levels
   double *sn = nullptr, *st = nullptr;   // [Ne] (hs_c2 - hs_c1)/d_e, (hs_v2 - hs_v1)/l_e
+  // FP64 states: cpd/2 sn ([Ne]); kappa_ce sn_e and kappa_ce st_e ([Nc][6])
+  double *hsn = nullptr, *ksnst = nullptr;
   // per cell and level [Nc][ld]: 1/dz, 1/dzh (interior half levels), upper interpolation
   // weight (interior half levels), reference Exner at the full level, dz
   double *inv_dz_c = nullptr, *inv_dzh_c = nullptr, *wu_c = nullptr, *exref_c = nullptr, *dz_c = nullptr;
@@ -174,6 +176,9 @@ struct StateDev {
   // 2 K_e, 2 rho_e vn and 4 rho_e vn theta_e at edges and folds the factors in here
   double *kin_w_h = nullptr, *div_wa_h = nullptr;
   double* adv_w = nullptr;             // kappa_ce / d_e ([Nc][3]): the FP64 step stores d_e a_e at edges
+  // per edge [Ne][4] 1/d_e, f_e, d_e/(6 l_e), -cpd/(2 d_e); per cell [Nc][4] the damping
+  // Laplacian's weights l_e/(A_c d_e) of the three neighbours and their sum (FP64 step)
+  double *edge_c = nullptr, *lap_w = nullptr;
   double *uvx = nullptr, *uvy = nullptr, *uvz = nullptr, *divc = nullptr, *thflx = nullptr;
   // mixed-mode scratch and shadows
   float *zeta32 = nullptr, *wv32 = nullptr, *vt32 = nullptr, *Ke32 = nullptr, *Kc32 = nullptr,

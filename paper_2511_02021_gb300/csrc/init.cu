@@ -259,6 +259,31 @@ __global__ void k_mixed_cells(int64_t nc, int64_t c0, int64_t n, int N, int ld, 
   }
 }
 
+// per-edge constants of the FP64 edge tendency
+__global__ void k_edge_consts(int64_t ne, const double* __restrict__ inv_de, const double* __restrict__ inv_le,
+                              const double* __restrict__ d_e, const double* __restrict__ f_e, double* __restrict__ out) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  out[4 * e] = inv_de[e];
+  out[4 * e + 1] = f_e[e];
+  out[4 * e + 2] = (inv_le[e] * d_e[e]) * (1.0 / 6.0);
+  out[4 * e + 3] = -0.5 * (kCpd * inv_de[e]);
+}
+
+// weights of the damping Laplacian: l_e / (A_c d_e) of the three neighbours, and their sum
+__global__ void k_lap_w(int64_t nc, const int* __restrict__ c2e, const double* __restrict__ div_wa,
+                        const double* __restrict__ inv_de, double* __restrict__ out) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= nc) return;
+  double sum = 0.0;
+  for (int s = 0; s < 3; ++s) {
+    const double w = fabs(div_wa[3 * c + s]) * inv_de[c2e[3 * c + s]];
+    out[4 * c + s] = w;
+    sum += w;
+  }
+  out[4 * c + 3] = sum;
+}
+
 // kappa_ce / d_e per cell and edge slot
 __global__ void k_adv_w(const double* __restrict__ kin_w, const int* __restrict__ c2e,
                         const double* __restrict__ inv_de, double* __restrict__ out, int64_t n) {
@@ -354,6 +379,8 @@ int init_state_device(icon_state* st, uint64_t seed, int case_id, const icon_cas
     k_half<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.kin_w, s.kin_w_h, 3 * g.nc);
     k_half<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.div_wa, s.div_wa_h, 3 * g.nc);
     k_adv_w<<<blocks_for(3 * g.nc, 256), 256, 0, stream>>>(g.kin_w, g.c2e, g.inv_de, s.adv_w, 3 * g.nc);
+    k_edge_consts<<<blocks_for(g.ne, 256), 256, 0, stream>>>(g.ne, g.inv_de, g.inv_le, g.d_e, g.f_e, s.edge_c);
+    k_lap_w<<<blocks_for(g.nc, 256), 256, 0, stream>>>(g.nc, g.c2e, g.div_wa, g.inv_de, s.lap_w);
     const TopoDev& T = s.topo;
     k_init_cells<<<blocks_for(g.nc, 128), 128, 0, stream>>>(cd, 0, g.nc, g.x_c, v.d_z_f, v.d_dzh, v.d_wu, v.d_wl,
                                                             T.on ? T.hs : nullptr, T.bf, T.wu_c, s.rho, s.thv,

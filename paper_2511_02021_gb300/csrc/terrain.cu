@@ -128,13 +128,26 @@ __global__ void k_topo_edges(LevelArgs L, int64_t ne, const int* __restrict__ e2
   }
 }
 
+// cpd/2 times the normal slope factor per edge; kappa_ce times both slope factors per cell
+__global__ void k_topo_slopes(int64_t nc, int64_t ne, const int* __restrict__ c2e, const double* __restrict__ kin_w,
+                              const double* __restrict__ sn, const double* __restrict__ st, double* __restrict__ hsn,
+                              double* __restrict__ ksnst) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < ne) hsn[i] = 0.5 * MUL(kCpd, sn[i]);
+  if (i >= nc) return;
+  for (int s = 0; s < 3; ++s) {
+    const int e = c2e[3 * i + s];
+    ksnst[6 * i + s] = MUL(kin_w[3 * i + s], sn[e]);
+    ksnst[6 * i + 3 + s] = MUL(kin_w[3 * i + s], st[e]);
+  }
+}
+
 struct StageArgs {
   int64_t nc;
   int N, ld;
   const int* c2e;
-  const double* kin_w;
   const double *vn, *vt, *w, *ex;             // stage state and its tangential velocity
-  const double *bf, *sn, *st;
+  const double *bf, *ksnst;
   const double *wu_c, *inv_dz_c, *inv_dzh_c, *exref_c;
   double *wcc, *wcon, *ep, *hdpdz;
 };
@@ -142,7 +155,7 @@ struct StageArgs {
 // one warp per cell, lanes over levels: the stage's contravariant correction and
 // contravariant velocity at half levels, the Exner perturbation and half its vertical
 // derivative at full levels. FP64-pipe bound like the step's stencils: the kappa and
-// slope factors of the three edges are combined once per cell (6 fused multiply-adds
+// slope factors of the three edges come combined from a table (6 fused multiply-adds
 // per full level), and the half-level interpolant takes the level above from the
 // neighbouring lane. Windows of 31 levels: lane l holds full level k = base + l and the
 // half level above it; lane 30's full level is carried to the next window.
@@ -154,11 +167,9 @@ __global__ void __launch_bounds__(256, 4) k_topo_cell(StageArgs a) {
   int64_t E[3];
   double An[3], At[3];
   for (int s = 0; s < 3; ++s) {
-    const int e = a.c2e[3 * c + s];
-    E[s] = (int64_t)e * ld;
-    const double kw = a.kin_w[3 * c + s];
-    An[s] = kw * a.sn[e];
-    At[s] = kw * a.st[e];
+    E[s] = (int64_t)a.c2e[3 * c + s] * ld;
+    An[s] = a.ksnst[6 * c + s];
+    At[s] = a.ksnst[6 * c + 3 + s];
   }
   double carry = 0.0;                       // X of the full level above the window
   for (int base = 0; base <= N; base += 31) {
@@ -318,6 +329,10 @@ int topo_build(icon_state* st, double h0, double radius, cudaStream_t stream) {
   for (double** p : cells) *p = A.get_n<double>(C);
   double** edges[] = {&T.wu_e, &T.qinv_dz_e, &T.dz_e};
   for (double** p : edges) *p = A.get_n<double>(E);
+  if (st->s.precision == ICON_FP64) {
+    T.hsn = A.get_n<double>(g.ne);
+    T.ksnst = A.get_n<double>(6 * (size_t)g.nc);
+  }
   if (A.failed) {
     set_error("out of device memory for the terrain-following metric tables");
     return ICON_ENOMEM;
@@ -338,6 +353,9 @@ int topo_build(icon_state* st, double h0, double radius, cudaStream_t stream) {
                                                                  T.exref_c, T.dz_c);
   k_topo_edges<<<blocks_for(g.ne * v.ld, 256), 256, 0, stream>>>(L, g.ne, g.e2c, g.e2v, g.v2c, g.vdeg, g.d_e, g.l_e,
                                                                  T.hs, T.wu_e, T.qinv_dz_e, T.dz_e, T.sn, T.st);
+  if (T.ksnst)
+    k_topo_slopes<<<blocks_for(g.ne > g.nc ? g.ne : g.nc, 256), 256, 0, stream>>>(g.nc, g.ne, g.c2e, g.kin_w, T.sn,
+                                                                                 T.st, T.hsn, T.ksnst);
   ICON_CUDA(cudaGetLastError());
   for (double* p : {T.wcc, T.wcon, T.ep, T.hdpdz}) ICON_CUDA(cudaMemsetAsync(p, 0, sizeof(double) * C, stream));
   if (st->s.precision == ICON_MIXED) {
@@ -383,9 +401,9 @@ void topo_stage(icon_state* st, const double* vn, const double* vt, const double
   const TopoDev& T = st->s.topo;
   StageArgs a;
   a.nc = g.nc; a.N = v.N; a.ld = v.ld;
-  a.c2e = g.c2e; a.kin_w = g.kin_w;
+  a.c2e = g.c2e;
   a.vn = vn; a.vt = vt; a.w = w; a.ex = ex;
-  a.bf = T.bf; a.sn = T.sn; a.st = T.st;
+  a.bf = T.bf; a.ksnst = T.ksnst;
   a.wu_c = T.wu_c; a.inv_dz_c = T.inv_dz_c; a.inv_dzh_c = T.inv_dzh_c; a.exref_c = T.exref_c;
   a.wcc = T.wcc; a.wcon = T.wcon; a.ep = T.ep; a.hdpdz = T.hdpdz;
   prof_begin(stream, K_TERRAIN);
