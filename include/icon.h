@@ -294,14 +294,14 @@ int icon_global_mass_noalloc(const icon_grid* grid, const double* dev_rho, const
 
 /* Copy a field (icon_field) to host memory as FP64, [entity][level] unpadded;
  * count must equal the field's element count. Synchronous. Pinned (page-locked) host
- * memory of a field stored in entity rows is written directly by the packing kernel over
- * the CPU-GPU link; other host memory goes through a device staging buffer and one copy. */
+ * memory is written directly by the packing kernel over the CPU-GPU link; other host
+ * memory goes through a device staging buffer and one copy. */
 int icon_state_copy_field(const icon_state* state, int field_id, double* host_dst, size_t count);
 
 /* Overwrite a prognostic field (ICON_F_VN .. ICON_F_EXNER) from FP64 host memory
  * in the same layout (rounded to FP32 where the state stores FP32). w at the lid
  * and the ground must be 0. Synchronous with respect to host_src. Pinned host memory
- * of a field stored in entity rows is read directly by the unpacking kernel. */
+ * is read directly by the unpacking kernel. */
 int icon_state_set_field(icon_state* state, int field_id, const double* host_src, size_t count);
 
 /* Number of kernel launches in the recorded graph of one step with the given
