@@ -301,7 +301,7 @@ int icon_state_copy_field(const icon_state* state, int field_id, double* host_ds
 /* Overwrite a prognostic field (ICON_F_VN .. ICON_F_EXNER) from FP64 host memory
  * in the same layout (rounded to FP32 where the state stores FP32). w at the lid
  * and the ground must be 0. Synchronous with respect to host_src. Pinned host memory
- * is read directly by the unpacking kernel. */
+ * of a field stored in entity rows is read directly by the unpacking kernel. */
 int icon_state_set_field(icon_state* state, int field_id, const double* host_src, size_t count);
 
 /* Number of kernel launches in the recorded graph of one step with the given

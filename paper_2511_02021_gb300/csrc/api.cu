@@ -452,7 +452,7 @@ __global__ void k_pack(const T* __restrict__ src, double* __restrict__ host, int
 // two orders cross in shared memory, so both sides are coalesced. Writing R2B6 / 90 levels (vn
 // and four level-major fields, 1.3 GB) to pinned memory took 33 ms with one word per thread in
 // device order, a row's stride apart in a staging buffer that was then copied; 6.9 ms now, a
-// field's 236 MB at 188 GB/s, the link's rate. Reading pinned memory this way: 108 GB/s.
+// field's 236 MB at 188 GB/s, the link's rate.
 constexpr int kPackThreads = 256;
 __global__ void __launch_bounds__(kPackThreads) k_pack_lm(const double* __restrict__ src, double* __restrict__ host,
                                                           int64_t n, int nlev) {
@@ -797,11 +797,12 @@ int icon_state_set_field(icon_state* st, int field_id, const double* host_src, s
     set_error("icon_state_set_field: field %d has %lld elements, got %zu", field_id, (long long)(n * nlev), count);
     return ICON_EINVAL;
   }
-  // pinned host memory is read by the unpack kernel directly, other memory through one
-  // contiguous transfer into a device buffer
+  // pinned host memory of a row-layout field is read by the unpack kernel directly; other memory
+  // goes through one contiguous transfer into a device buffer (as do level-major fields from
+  // pinned memory: the kernel's own reads over the link reach 108 GB/s, the transfer 207)
   const int ld = st->grid->vert.ld;
   cudaStream_t stream = current_stream();
-  double* hs = const_cast<double*>(static_cast<const double*>(mapped_host_ptr(host_src)));
+  double* hs = lm ? nullptr : const_cast<double*>(static_cast<const double*>(mapped_host_ptr(host_src)));
   DeviceArena tmp;
   tmp.al = st->arena.al;
   double* stage = hs ? hs : tmp.get_n<double>((size_t)n * nlev);

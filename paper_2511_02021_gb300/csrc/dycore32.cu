@@ -280,11 +280,6 @@ __device__ inline void mx_dd_edge_item(const MxGeo& G, const MxDDArgs& a, int64_
   }
 }
 
-__global__ void __launch_bounds__(256) k_mx_dd_edge(MxGeo G, MxDDArgs a) {
-  const int64_t e = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (e < G.ne) mx_dd_edge_item(G, a, e, threadIdx.x & 31);
-}
-
 // diffusion: least-squares vertex velocity and O3 curl of vn
 template <int LPE>
 __device__ inline void mx_diff_vertex_item(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ ux,
@@ -1697,18 +1692,11 @@ void with_lanes(int lanes, F f) {
   else f(std::integral_constant<int, 32>{});
 }
 
-// the lean gather: blocks of at most 256 threads (32 groups of eight lanes, one per cell)
 template <bool CORR>
-void launch_lean_gather(const MxGeo& G, const MxLeanArgs& a, bool fused, bool topo, int block, cudaStream_t st) {
+void launch_lean_gather(const MxGeo& G, const MxLeanArgs& a, bool topo, cudaStream_t st) {
   const unsigned nb = blocks_for(G.nc, 32);
-  const int B = block < 256 ? block : 256;
-  if (CORR && fused) {
-    if (topo) k_mx_lean_gather<CORR, CORR, true><<<nb, B, 0, st>>>(G, a);
-    else k_mx_lean_gather<CORR, CORR, false><<<nb, B, 0, st>>>(G, a);
-  } else {
-    if (topo) k_mx_lean_gather<CORR, false, true><<<nb, B, 0, st>>>(G, a);
-    else k_mx_lean_gather<CORR, false, false><<<nb, B, 0, st>>>(G, a);
-  }
+  if (topo) k_mx_lean_gather<CORR, true><<<nb, 256, 0, st>>>(G, a);
+  else k_mx_lean_gather<CORR, false><<<nb, 256, 0, st>>>(G, a);
 }
 
 void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, const MxEdgeArgs& ea,
@@ -1736,6 +1724,7 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
     case K_MX_EDGE_TEND:
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
+        const int B = t.block < 256 ? t.block : 256;       // 85 registers for three such blocks per SM
         if (s.topo.on) k_mx_edge_tend<LPE, true><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
         else k_mx_edge_tend<LPE, false><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
       });
@@ -1749,10 +1738,6 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
       break;
     case K_MX_COLUMN_PREP: {   // the predictor's gather (the corrector's only differs in the Aw0 average)
       const unsigned nb = (unsigned)((G.nc + 31) / 32);
-      if (s.ln_B) {
-        launch_lean_gather<false>(G, lean_args(s, false, (double)ea.dtau, 1), false, s.topo.on, B, st);
-        break;
-      }
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
         k_mx_gather_tile<LPE, false><<<nb, B, 0, st>>>(G, ca);
@@ -1789,7 +1774,8 @@ void launch_mx_column(const MxGeo& G, const MxColArgs& a, bool topo, cudaStream_
 // ---------------------------------------------------------------- autotuner
 // Candidate tiles over (entity, level): 32 lanes per entity (one entity per warp), 16
 // (two per warp) or 8 (four per warp), blocks of 64, 128, 256 or 512 threads: twelve per
-// stencil kind. (The lean column's form follows a rule on the grid's size, lean_form.) Each kind is timed on the state's own data (three launches
+// stencil kind. (The lean column's form follows a rule on the grid's size, lean_form, and its
+// gather has one shape.) Each kind is timed on the state's own data (three launches
 // per candidate after one untimed, CUDA events) and the fastest kept, in the order of the
 // step, so that every trial reads inputs its predecessors formed. Choices are cached per
 // (kind, grid size, levels, GPU) in the process and, if the environment variable
@@ -1847,15 +1833,11 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   const MxEdgeArgs ea = edge_args(s, false, dtau, nsub);
   const MxColArgs ca = col_args(s, false, dtau, nsub);
   const bool lean = s.ln_B != nullptr;
-  if (lean) {
-    // the lean gather's weights for this dtau, so that its trials compute on valid inputs
-    k_mx_dwa_t<<<blocks_for(G.nc, 256), 256, 0, stream>>>(G.nc, G.div_wa, G.inv_Ac, dtau, s.ln_dwa, s.ln_cw32);
-  }
   std::lock_guard<std::mutex> lk(g_tune_mu);
   load_tune_file();
   for (int kind : kTunedKinds) {
     if (st->tile[kind].lanes != 0 && st->tile_forced[kind]) continue;
-    if (kind == K_MX_COLUMN_PREP && !s.fac64 && !lean) continue;
+    if (kind == K_MX_COLUMN_PREP && !s.fac64) continue;
     const std::string key = tune_key(kind, G);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
@@ -1864,9 +1846,7 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
     }
     std::vector<TileChoice> cands;
     for (int lanes : kTileLanes)
-      for (int block : kTileBlocks)
-        if (!(kind == K_MX_COLUMN_PREP && lean) || (lanes == 8 && block <= 256))   // the lean gather's lanes are fixed
-          cands.push_back(TileChoice{lanes, block});
+      for (int block : kTileBlocks) cands.push_back(TileChoice{lanes, block});
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -1891,7 +1871,9 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   // a trial that met a non-finite value would have flagged the state; the step that
   // follows checks it again
   cudaMemsetAsync(s.status, 0, sizeof(unsigned), stream);
+  // the lean column's form follows the grid's size and its gather has one shape
   if (lean && !st->tile_forced[K_MX_LEAN]) st->tile[K_MX_LEAN] = kLeanDefault;
+  if (lean && !st->tile_forced[K_MX_COLUMN_PREP]) st->tile[K_MX_COLUMN_PREP] = TileChoice{8, 256};
   st->tuned = true;
 }
 
@@ -1911,7 +1893,7 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
   }
   auto tile = [&](int kind) { return st->tile[kind].lanes ? st->tile[kind] : TileChoice{32, 256}; };
   // The next stage's edge diagnostics (vt) and cell kinetic energy read only that stage's vn,
-  // final once this stage's edge tendency (predictor) or damped gather (corrector) has run,
+  // final once this stage's edge tendency (predictor) or damping (corrector) has run,
   // and write vt32 and Kc32, which neither this stage's gather nor its column reads. While a
   // step on flat levels is recorded into its graph they go on a second branch beside the
   // column, whose last wave of blocks leaves part of the SMs idle; the branch is joined before
@@ -1942,14 +1924,9 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
       const MxEdgeArgs ea = edge_args(s, corr, dtau, nsub);
       const MxColArgs ca = col_args(s, corr, dtau, nsub);
       const bool damp = corr && st->divdamp4 > 0.0;
-      // lean column with damping: the corrector's undamped vn^{n+1} goes to Avn0_32 (dead once
-      // the edge tendency has read it, element by element), the damping's edge update is
-      // formed inside the gather, which writes the damped vn^{n+1} and the step-mean flux
-      const bool fused = lean && damp;
       MxEdgeArgs ead = ea;
       ead.skip_flux = damp ? 1 : 0;
       ead.upwind_theta = st->upwind_theta ? 1 : 0;
-      if (fused) ead.vn_out = s.Avn0_32;
       for (int kind : {K_MX_VERTEX, K_MX_EDGE, K_MX_CELL_KE, K_MX_EDGE_TEND}) {
         if (diag_ahead && (kind == K_MX_EDGE || kind == K_MX_CELL_KE)) continue;
         if (diag_ahead && kind == K_MX_EDGE_TEND) {
@@ -1971,25 +1948,18 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
         da.vn = s.vn32; da.phi = s.F32; da.gth = s.G32; da.mflx = s.mflx;
         da.scale = (float)(st->divdamp4 * abar * abar); da.inv_nsub = 1.0 / nsub;
         da.upwind_theta = st->upwind_theta ? 1 : 0;
-        const unsigned nbq = item_blocks(nc, kQuadLanes, 256), nbe8 = (unsigned)((G.ne + 7) / 8);
+        const unsigned nbq = item_blocks(nc, kQuadLanes, 256);
         prof_begin(stream, K_DIVDAMP);
-        k_mx_dd_div<<<nbq, 256, 0, stream>>>(G, fused ? s.Avn0_32 : s.vn32, s.Kc32);
+        k_mx_dd_div<<<nbq, 256, 0, stream>>>(G, s.vn32, s.Kc32);
         k_mx_dd_lap<<<nbq, 256, 0, stream>>>(G, s.Kc32, s.vt32);
-        if (!fused) k_mx_dd_edge<<<nbe8, 256, 0, stream>>>(G, da);
+        k_mx_dd_edge<<<item_blocks(G.ne, kQuadLanes, 256), 256, 0, stream>>>(G, da);
         prof_end(stream);
       }
       if (lean) {
-        MxLeanArgs la = lean_args(s, corr, dtau, nsub);
-        if (fused) {
-          la.dd_vn = s.Avn0_32; la.dd_L = s.vt32; la.dd_rho = ea.rho; la.dd_thv = ea.thv;
-          la.dd_out = s.vn32; la.mflx = s.mflx;
-          la.dd_scale = (float)(st->divdamp4 * st->abar * st->abar);
-          la.dd_upwind = st->upwind_theta ? 1 : 0;
-        }
-        const int block = tile(K_MX_COLUMN_PREP).block;
+        const MxLeanArgs la = lean_args(s, corr, dtau, nsub);
         prof_begin(stream, K_MX_LEAN_GATHER);
-        if (corr) launch_lean_gather<true>(G, la, fused, s.topo.on, block, stream);
-        else launch_lean_gather<false>(G, la, false, s.topo.on, block, stream);
+        if (corr) launch_lean_gather<true>(G, la, s.topo.on, stream);
+        else launch_lean_gather<false>(G, la, s.topo.on, stream);
         prof_end(stream);
         if (overlap && (!corr || it + 1 < nsub)) fork_diag(!corr);
         prof_begin(stream, K_MX_LEAN);

@@ -26,6 +26,19 @@ __device__ __forceinline__ void fma4(F4& acc, float w, const F4& x) {
   for (int i = 0; i < 4; ++i) acc.v[i] = __fmaf_rn(w, x.v[i], acc.v[i]);
 }
 
+// m += w x on a quad of an FP64 row (whole 16-byte words: element by element, every store wrote a
+// quarter of each 32-byte sector it touched)
+__device__ __forceinline__ void add4(double* m, const F4& x, double w) {
+  double2* q = reinterpret_cast<double2*>(m);
+  double2 a = q[0], b = q[1];
+  a.x = __fma_rn(f32_to_f64(x.v[0]), w, a.x);
+  a.y = __fma_rn(f32_to_f64(x.v[1]), w, a.y);
+  b.x = __fma_rn(f32_to_f64(x.v[2]), w, b.x);
+  b.y = __fma_rn(f32_to_f64(x.v[3]), w, b.y);
+  q[0] = a;
+  q[1] = b;
+}
+
 // warp w, lanes [sub*LPE, (sub+1)*LPE) handle entity w * (32/LPE) + sub
 #define QUAD_PROLOGUE(LPE, COUNT)                                                        \
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;             \
@@ -128,7 +141,7 @@ __global__ void __launch_bounds__(512) k_mx_cell_ke(MxGeo G, const float* __rest
 // the metric correction of the pressure gradient (exp is then against the per-cell reference),
 // fluxes through dz_e.
 template <int LPE, bool TOPO>
-__global__ void __launch_bounds__(512, 1) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
+__global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
   QUAD_PROLOGUE(LPE, G.ne)
   const int64_t e = item;
   const int ld = G.ld, N = G.N, nh = (N + 4) >> 2;
@@ -238,16 +251,12 @@ __global__ void __launch_bounds__(512, 1) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) 
     }
     st4(phi_o + k0, F);
     st4(gth_o + k0, g);
-    if (corr) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (k0 + i < N) mflx_o[k0 + i] += f32_to_f64(F.v[i]) * inv_nsub;
-    }
+    if (corr) add4(mflx_o + k0, F, inv_nsub);
   }
 }
 
-// ---- fourth-order divergence damping of the corrector's vn^{n+1}: cell divergence, then its
-// cell Laplacian (eight lanes per cell, four cells per warp)
+// ---- fourth-order divergence damping of the corrector's vn^{n+1}: cell divergence, its cell
+// Laplacian, then the edge update (eight lanes per entity, four entities per warp)
 constexpr int kQuadLanes = 8;
 
 __global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restrict__ vn, float* __restrict__ D) {
@@ -297,6 +306,37 @@ __global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restr
       l.v[i] = wt[0] * g0 + wt[1] * g1 + wt[2] * g2;
     }
     st4(L + c * ld + 4 * q, l);
+  }
+}
+
+// the damping's edge update with the corrector's fluxes and the FP64 step-mean mass flux. A kernel
+// of its own: formed inside the corrector's gather by both cells of every edge, it saved the
+// fluxes' round trip but held so many neighbour rows that the gather spilled at 64 registers and
+// waited on its loads at 80. R2B6/90, per step: gather 4.63 and damping 0.64 ms with it fused,
+// 2.72 and 2.25 ms apart (this kernel 322 us per launch, 5.5 TB/s of its 60 B per cell-level)
+__global__ void __launch_bounds__(256, 4) k_mx_dd_edge(MxGeo G, MxDDArgs a) {
+  QUAD_PROLOGUE(kQuadLanes, G.ne)
+  const int64_t e = item;
+  const int ld = G.ld, nq = (G.N + 3) >> 2;
+  const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld, o = e * ld;
+  const float sc = a.scale * G.inv_de32[e], le = G.l_e32[e];
+  for (int q = lane; q < nq; q += kQuadLanes) {
+    const int k = 4 * q;
+    const F4 v = ld4(a.vn + o + k), L1 = ld4(a.L + c1 + k), L2 = ld4(a.L + c2 + k);
+    const F4 r1 = ld4(a.rho + c1 + k), r2 = ld4(a.rho + c2 + k), t1 = ld4(a.thv + c1 + k), t2 = ld4(a.thv + c2 + k);
+    F4 dz{}, vd, F, g;
+    if (a.dz_e) dz = ld4(a.dz_e + o + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      vd.v[i] = __fmaf_rn(-sc, L2.v[i] - L1.v[i], v.v[i]);
+      F.v[i] = 0.5f * (r1.v[i] + r2.v[i]) * vd.v[i];
+      if (a.dz_e) F.v[i] *= dz.v[i];
+      g.v[i] = (le * F.v[i]) * (a.upwind_theta ? (vd.v[i] >= 0.0f ? t1.v[i] : t2.v[i]) : 0.5f * (t1.v[i] + t2.v[i]));
+    }
+    st4(a.vn + o + k, vd);
+    st4(a.phi + o + k, F);
+    st4(a.gth + o + k, g);
+    add4(a.mflx + o + k, F, a.inv_nsub);
   }
 }
 
@@ -467,84 +507,41 @@ __global__ void __launch_bounds__(256, 4) k_mx_diff_theta(MxGeo G, const float* 
 // ---- gather of the lean column's stage inputs: a block takes 32 consecutive cells, eight lanes
 // per cell gather its edges by quads of levels (32 levels per pass), and the results cross to
 // level-major order through shared memory (32 consecutive cells per level). CORR: the
-// predictor's A_w is averaged in as the rows are written, where it is read coalesced. DDF: the
-// divergence damping's edge update fused in; each cell's own rows of the Laplacian, rho and
-// theta_v are loaded once and serve its three edges; the lower-id cell of an edge stores the
-// damped vn and accumulates the step-mean flux. TOPO (terrain-following levels): fluxes through
-// the edges' layer thickness, the vertical advection of w with w - wcc and the cell's own 1/dzh;
+// predictor's A_w is averaged in as the rows are written, where it is read coalesced. TOPO
+// (terrain-following levels): the vertical advection of w with w - wcc and the cell's own 1/dzh;
 // the divergences stay per unit thickness and the column scales them by the cell's 1/dz.
-template <bool CORR, bool DDF, bool TOPO>
-__global__ void __launch_bounds__(256, 3) k_mx_lean_gather(MxGeo G, MxLeanArgs a) {
+template <bool CORR, bool TOPO>
+__global__ void __launch_bounds__(256, 4) k_mx_lean_gather(MxGeo G, MxLeanArgs a) {
   __shared__ double sd[CORR ? 32 : 1][33];
   __shared__ float sf[CORR ? 2 : 3][32][33];                 // dtau D_Theta, A_w, dtau D_rho (predictor)
   const int N = G.N, ld = G.ld;
   const int64_t nc = G.nc, c0 = (int64_t)blockIdx.x * 32;
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 7, ngrp = nthr >> 3;
+  const int tid = threadIdx.x, lane = tid & 7, cl = tid >> 3;
   const float dtau32 = (float)a.dtau;
+  // the cell's neighbours and weights, held for every pass over the levels
+  const bool act = c0 + cl < nc;
+  const int64_t c = act ? c0 + cl : 0, o = c * ld;
+  const float4 cw = a.cw32[c];
+  int64_t E[3];
+  float sg[3], kw[3];
+  double dwt[3];
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    E[s] = (int64_t)G.c2e[3 * c + s] * ld;
+    sg[s] = G.s_ce32[3 * c + s];
+    kw[s] = G.kin_w32[3 * c + s];
+    if (CORR) dwt[s] = a.dwa_t[3 * c + s];
+  }
   for (int k0 = 0; k0 < N; k0 += 32) {
     const int k = k0 + 4 * lane;
-    for (int cl = tid >> 3; cl < 32; cl += ngrp) {
-      const int64_t c = c0 + cl;
-      if (c >= nc || k >= N) break;
-      const int64_t o = c * ld;
-      const float4 cw = a.cw32[c];
-      const float dw32[3] = {cw.x, cw.y, cw.z};
-      F4 ae[3], D{}, T{};
-      double Dd[4] = {0.0, 0.0, 0.0, 0.0};
-      F4 F[3], Gt[3];
-      F4 Lm{}, rm{}, tm{};
-      if constexpr (DDF) {
-        Lm = ld4(a.dd_L + o + k);
-        rm = ld4(a.dd_rho + o + k);
-        tm = ld4(a.dd_thv + o + k);
-      }
+    if (act && k < N) {
+      F4 ae[3], F[3], Gt[3];
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
-        const int e = G.c2e[3 * c + s];
-        const int64_t E = (int64_t)e * ld + k;
-        ae[s] = ld4(a.a_e + E);
-        if constexpr (DDF) {
-          // damped vn^{n+1} and its fluxes, as the damping's edge update forms them
-          const int ca = G.e2c[2 * e], cb = G.e2c[2 * e + 1];
-          const bool own = ca == c;
-          const int64_t nb = (int64_t)(own ? cb : ca) * ld + k;
-          const float sc = a.dd_scale * G.inv_de32[e], le = G.l_e32[e];
-          const F4 v = ld4(a.dd_vn + E), Ln = ld4(a.dd_L + nb), rn = ld4(a.dd_rho + nb), tn = ld4(a.dd_thv + nb);
-          F4 dz{}, vd;
-          if constexpr (TOPO) dz = ld4(a.t_dz_e + E);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float dL = own ? Ln.v[i] - Lm.v[i] : Lm.v[i] - Ln.v[i];
-            vd.v[i] = __fmaf_rn(-sc, dL, v.v[i]);
-            float f = 0.5f * (rm.v[i] + rn.v[i]) * vd.v[i];
-            if constexpr (TOPO) f *= dz.v[i];
-            const float t1 = own ? tm.v[i] : tn.v[i], t2 = own ? tn.v[i] : tm.v[i];
-            F[s].v[i] = f;
-            Gt[s].v[i] = (le * f) * (a.dd_upwind ? (vd.v[i] >= 0.0f ? t1 : t2) : 0.5f * (t1 + t2));
-          }
-          if (own) {
-            st4(a.dd_out + E, vd);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (k + i < N) a.mflx[E + i] += (double)F[s].v[i] * a.inv_nsub;
-          }
-        } else {
-          F[s] = ld4(a.phi + E);
-          Gt[s] = ld4(a.gth + E);
-        }
+        ae[s] = ld4(a.a_e + E[s] + k);
+        F[s] = ld4(a.phi + E[s] + k);
+        Gt[s] = ld4(a.gth + E[s] + k);
       }
-      const float sg0 = G.s_ce32[3 * c], sg1 = G.s_ce32[3 * c + 1], sg2 = G.s_ce32[3 * c + 2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        // the hardware conversion here: the gather leaves the FP64 pipe half idle, and the
-        // integer-pipe form costs more issue slots
-        if (CORR)
-          Dd[i] = (a.dwa_t[3 * c] * (double)F[0].v[i] + a.dwa_t[3 * c + 1] * (double)F[1].v[i]) +
-                  a.dwa_t[3 * c + 2] * (double)F[2].v[i];
-        else D.v[i] = (dw32[0] * F[0].v[i] + dw32[1] * F[1].v[i]) + dw32[2] * F[2].v[i];
-        T.v[i] = (sg0 * Gt[0].v[i] + sg1 * Gt[1].v[i] + sg2 * Gt[2].v[i]) * cw.w;
-      }
-      const float kw0 = G.kin_w32[3 * c], kw1 = G.kin_w32[3 * c + 1], kw2 = G.kin_w32[3 * c + 2];
       const F4 w = ld4(a.w_stage + o + k);
       const float wm = k > 0 ? a.w_stage[o + k - 1] : 0.0f, wp = k + 4 <= N ? a.w_stage[o + k + 4] : 0.0f;
       F4 wc{}, iz;
@@ -556,29 +553,33 @@ __global__ void __launch_bounds__(256, 3) k_mx_lean_gather(MxGeo G, MxLeanArgs a
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float hadv = kw0 * ae[0].v[i] + kw1 * ae[1].v[i] + kw2 * ae[2].v[i];
+        const int r = 4 * lane + i;
+        // conversions on the integer pipe: the hardware ones are FP64-pipe operations, a warp
+        // instruction per SM every 16 cycles
+        if (CORR)
+          sd[r][cl] = (dwt[0] * f32_to_f64(F[0].v[i]) + dwt[1] * f32_to_f64(F[1].v[i])) + dwt[2] * f32_to_f64(F[2].v[i]);
+        else
+          sf[2][r][cl] = (cw.x * F[0].v[i] + cw.y * F[1].v[i]) + cw.z * F[2].v[i];
+        sf[0][r][cl] = (sg[0] * Gt[0].v[i] + sg[1] * Gt[1].v[i] + sg[2] * Gt[2].v[i]) * cw.w;
+        const float hadv = kw[0] * ae[0].v[i] + kw[1] * ae[1].v[i] + kw[2] * ae[2].v[i];
         const float wu = i ? w.v[i ? i - 1 : 0] : wm, wd = i < 3 ? w.v[i < 3 ? i + 1 : 3] : wp;
         float Aw;
         if constexpr (TOPO) Aw = -hadv - wc.v[i] * (wu - wd) * (0.5f * iz.v[i]);
         else Aw = -hadv - w.v[i] * (wu - wd) * iz.v[i];
-        const int r = 4 * lane + i;
-        if (CORR) sd[r][cl] = Dd[i];
-        else sf[2][r][cl] = D.v[i];
-        sf[0][r][cl] = T.v[i];
         sf[1][r][cl] = Aw;
       }
     }
     __syncthreads();
-    for (int i = tid; i < 32 * 32; i += nthr) {
-      const int r = i >> 5, cl = i & 31, kk = k0 + r;
-      const int64_t c = c0 + cl;
-      if (c >= nc || kk >= N) continue;
-      const int64_t j = (int64_t)kk * nc + c;
-      if (CORR) a.dr64[j] = sd[r][cl];
-      else a.dr32[j] = sf[2][r][cl];
-      a.dt32[j] = sf[0][r][cl];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = (tid >> 5) + 8 * i, ci = tid & 31, kk = k0 + r;
+      if (c0 + ci >= nc || kk >= N) continue;
+      const int64_t j = (int64_t)kk * nc + c0 + ci;
+      if (CORR) a.dr64[j] = sd[r][ci];
+      else a.dr32[j] = sf[2][r][ci];
+      a.dt32[j] = sf[0][r][ci];
       if (kk >= 1) {
-        float Aw = sf[1][r][cl];
+        float Aw = sf[1][r][ci];
         if (CORR) Aw = 0.5f * (a.Aw0[j] + Aw);
         else a.Aw0[j] = Aw;
         a.aw32[j] = dtau32 * Aw;
