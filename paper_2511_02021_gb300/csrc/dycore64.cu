@@ -62,6 +62,7 @@ struct Geo64 {
   // [Ne][4] 1/d_e, f_e, d_e / (6 l_e), -cpd / (2 d_e); per cell [Nc][4] the damping Laplacian's
   // weights l_e / (A_c d_e) of the three neighbours and their sum
   const double4 *edge_c, *lap_w;
+  bool merge_column, merge_stencil;        // the global grid takes the merged launches
   // terrain-following levels (the TOPO kernel variants; see terrain.cu): per-edge normal
   // slope factor times cpd / 2, full-level decay, per-entity tables [entity][ld], and the stage's
   // contravariant correction, contravariant velocity, Exner perturbation and half its
@@ -105,9 +106,8 @@ __device__ inline int64_t warp_entity() {
 
 // zeta_v (full levels) and six times w_v (half levels): the plain sum of a hexagon's cells,
 // scaled by 6/5 at the twelve pentagons (the 1/6 is in the edge tendency's per-edge constant)
-__global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __restrict__ vn, const double* __restrict__ w,
-                                                double* __restrict__ zeta, double* __restrict__ w_v) {
-  const int64_t v = warp_entity();
+__device__ __forceinline__ void vertex_item(const Geo64& G, const double* __restrict__ vn, const double* __restrict__ w,
+                                            double* __restrict__ zeta, double* __restrict__ w_v, int64_t v) {
   if (v >= G.nv) return;
   const int lane = threadIdx.x & 31, ld = G.ld;
   int64_t E[6], C[6];
@@ -133,9 +133,8 @@ __global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __rest
 }
 
 // vt (Perot) and 2 K_e = vn^2 + vt^2 at edges (the 1/2 is folded into k_cell_ke's weights)
-__global__ void __launch_bounds__(256) k_edge_vt(Geo64 G, const double* __restrict__ vn, double* __restrict__ vt,
-                                                 double* __restrict__ Ke) {
-  const int64_t e = warp_entity();
+__device__ __forceinline__ void edge_vt_item(const Geo64& G, const double* __restrict__ vn, double* __restrict__ vt,
+                                             double* __restrict__ Ke, int64_t e) {
   if (e >= G.ne) return;
   const int lane = threadIdx.x & 31, ld = G.ld;
   int64_t S[5];
@@ -151,6 +150,26 @@ __global__ void __launch_bounds__(256) k_edge_vt(Geo64 G, const double* __restri
     vt[e * ld + k] = acc;
     Ke[e * ld + k] = fma(v0, v0, acc * acc);
   }
+}
+
+__global__ void __launch_bounds__(256, 4) k_vertex(Geo64 G, const double* __restrict__ vn, const double* __restrict__ w,
+                                                double* __restrict__ zeta, double* __restrict__ w_v) {
+  vertex_item(G, vn, w, zeta, w_v, warp_entity());
+}
+
+__global__ void __launch_bounds__(256) k_edge_vt(Geo64 G, const double* __restrict__ vn, double* __restrict__ vt,
+                                                 double* __restrict__ Ke) {
+  edge_vt_item(G, vn, vt, Ke, warp_entity());
+}
+
+// both, on small grids: neither reads what the other writes, and a launch there costs more than
+// the work (the first nbv blocks take the vertices)
+__global__ void __launch_bounds__(256, 4) k_vertex_edge_vt(Geo64 G, const double* __restrict__ vn,
+                                                        const double* __restrict__ w, double* __restrict__ zeta,
+                                                        double* __restrict__ w_v, double* __restrict__ vt,
+                                                        double* __restrict__ Ke, unsigned nbv) {
+  if (blockIdx.x < nbv) vertex_item(G, vn, w, zeta, w_v, warp_entity());
+  else edge_vt_item(G, vn, vt, Ke, warp_entity() - (int64_t)nbv * kWarpsPerBlock);
 }
 
 // K_c at cells (from 2 K_e)
@@ -355,7 +374,7 @@ __global__ void __launch_bounds__(256, 4) k_dd_edge(Geo64 G, DDArgs a) {
 // ---------------------------------------------------------------- column solve
 //
 // The vertically implicit update of every column in three launches:
-//   k_col_rows_*  one warp per cell, lanes over levels: everything that is parallel
+//   k_col_rows   one warp per cell, lanes over levels: everything that is parallel
 //                over the levels (half-level interpolants, horizontal divergences,
 //                explicit predictors, the linearised state equation, the w predictor
 //                and, in the predictor, the tridiagonal row of every interior half
@@ -414,9 +433,7 @@ struct ColArgs {
 // the explicit vertical fluxes with the contravariant (1 - beta) w - wcc, and the
 // vertical advection of w with w - wcc; S^n stays, since those fluxes change with the stage.
 template <bool TOPO>
-__global__ void __launch_bounds__(256, 4) k_col_rows_pred(Geo64 G, ColArgs a) {
-  const int64_t c = warp_entity();
-  if (c >= G.nc) return;
+__device__ __forceinline__ void col_rows_pred(const Geo64& G, const ColArgs& a, int64_t c) {
   const int lane = threadIdx.x & 31, ld = G.ld, N = G.N;
   const int64_t o = c * ld, nc = G.nc;
   const double* __restrict__ cc = G.cc;
@@ -546,9 +563,7 @@ __global__ void __launch_bounds__(256, 4) k_col_rows_pred(Geo64 G, ColArgs a) {
 // the corrector's right-hand side and explicit parts, from what the predictor left. Flat levels
 // need the level above only: windows of 32 with lane 31's carried.
 template <bool TOPO>
-__global__ void __launch_bounds__(256, 4) k_col_rows_corr(Geo64 G, ColArgs a) {
-  const int64_t c = warp_entity();
-  if (c >= G.nc) return;
+__device__ __forceinline__ void col_rows_corr(const Geo64& G, const ColArgs& a, int64_t c) {
   const int lane = threadIdx.x & 31, ld = G.ld, N = G.N;
   const int64_t o = c * ld, nc = G.nc;
   int64_t E[3];
@@ -614,17 +629,13 @@ __global__ void __launch_bounds__(256, 4) k_col_rows_corr(Geo64 G, ColArgs a) {
 // 1 / pivot over the diagonal and up / pivot over the super-diagonal, and the corrector only
 // substitutes its own right-hand side. The damped solution goes over the right-hand side.
 template <bool CORR>
-__global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= G.nc) return;
+__device__ __forceinline__ void col_thomas(const Geo64& G, const ColArgs& a, int64_t c) {
   const int N = G.N, ld = G.ld;
   if (N < 2) return;
   const int64_t nc = G.nc;
   const double* __restrict__ cc = G.cc;
-  const double* __restrict__ lo = a.lo;
-  double* __restrict__ di = a.di;
-  double* __restrict__ up = a.up;
-  double* __restrict__ rh = a.rh;
+  const double* lo = a.lo;
+  double *di = a.di, *up = a.up, *rh = a.rh;
   double dp = 0.0;
   if (!CORR) {
     double cp = 0.0;
@@ -670,9 +681,7 @@ __global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
 // TOPO: each cell's dz, the contravariant step-mean vertical flux, and the ground w of
 // the stage (its wcc, so that w - wcc = 0 there)
 template <bool TOPO, bool CORR>
-__global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
-  const int64_t c = warp_entity();
-  if (c >= G.nc) return;
+__device__ __forceinline__ void col_update(const Geo64& G, const ColArgs& a, int64_t c) {
   const int lane = threadIdx.x & 31, ld = G.ld, N = G.N;
   const int64_t o = c * ld, nc = G.nc;
   const double* __restrict__ cc = G.cc;
@@ -710,6 +719,45 @@ __global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
   }
   if (lane == 0) a.w_o[o + N] = TOPO ? G.t_wcc[o + N] : 0.0;
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, 1u);
+}
+
+template <bool TOPO, bool CORR>
+__device__ __forceinline__ void col_rows(const Geo64& G, const ColArgs& a, int64_t c) {
+  if constexpr (CORR) col_rows_corr<TOPO>(G, a, c);
+  else col_rows_pred<TOPO>(G, a, c);
+}
+
+template <bool TOPO, bool CORR>
+__global__ void __launch_bounds__(256, 4) k_col_rows(Geo64 G, ColArgs a) {
+  const int64_t c = warp_entity();
+  if (c < G.nc) col_rows<TOPO, CORR>(G, a, c);
+}
+
+template <bool CORR>
+__global__ void __launch_bounds__(128) k_col_thomas(Geo64 G, ColArgs a) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c < G.nc) col_thomas<CORR>(G, a, c);
+}
+
+template <bool TOPO, bool CORR>
+__global__ void __launch_bounds__(256) k_col_update(Geo64 G, ColArgs a) {
+  const int64_t c = warp_entity();
+  if (c < G.nc) col_update<TOPO, CORR>(G, a, c);
+}
+
+// the three in one launch, on small grids: a block takes eight cells, one per warp in the
+// level-parallel parts, and eight lanes walk their columns; the rows pass through global memory
+// (the block's own barriers order them) and stay in L2. Eight cells and not 32: an SM's FP64 pipe
+// takes a warp instruction every 16 cycles, so a small grid has to be spread over all SMs
+// (R2B2/20: 450 us per step with 32 cells a block, 356 with eight).
+template <bool TOPO, bool CORR>
+__global__ void __launch_bounds__(256, 4) k_col_small(Geo64 G, ColArgs a) {
+  const int64_t c0 = (int64_t)blockIdx.x * kWarpsPerBlock, c = warp_entity();
+  if (c < G.nc) col_rows<TOPO, CORR>(G, a, c);
+  __syncthreads();
+  if (threadIdx.x < kWarpsPerBlock && c0 + threadIdx.x < G.nc) col_thomas<CORR>(G, a, c0 + threadIdx.x);
+  __syncthreads();
+  if (c < G.nc) col_update<TOPO, CORR>(G, a, c);
 }
 
 // ---------------------------------------------------------------- diffusion
@@ -874,23 +922,34 @@ Geo64 make_geo(const icon_grid* grid, const double* cc) {
   G.cc = cc;
   G.kin_w_h = G.div_wa_h = G.adv_w = nullptr;
   G.edge_c = G.lap_w = nullptr;
+  G.merge_column = G.merge_stencil = false;
   G.t_hsn = G.t_bf = G.t_wu_e = G.t_qinv_dz_e = G.t_dz_e = nullptr;
   G.t_wu_c = G.t_inv_dz_c = G.t_inv_dzh_c = G.t_wcc = G.t_wcon = G.t_ep = G.t_hdpdz = nullptr;
   return G;
 }
 
+// Merged launches on small grids, whose kernels run 2 to 4 us, about what starting one takes: the
+// column's three parts up to R2B2 (1,280 cells; 90 launches per step of R2B2/20 398 us, merged 356;
+// on R2B3/90 the parts fill the SMs better apart, 2334 against 2887 us), vertices with edges up
+// to R2B3.
+constexpr int64_t kMergeColumnCells = 1280, kMergeStencilCells = 5120;
+
+template <bool TOPO, bool CORR>
+void launch_column_as(const Geo64& G, const ColArgs& a, cudaStream_t st) {
+  if (G.merge_column) {
+    k_col_small<TOPO, CORR><<<blocks_for(G.nc, kWarpsPerBlock), 256, 0, st>>>(G, a);
+    return;
+  }
+  const unsigned nbc = blocks_for(G.nc, kWarpsPerBlock);
+  k_col_rows<TOPO, CORR><<<nbc, 256, 0, st>>>(G, a);
+  k_col_thomas<CORR><<<blocks_for(G.nc, 128), 128, 0, st>>>(G, a);
+  k_col_update<TOPO, CORR><<<nbc, 256, 0, st>>>(G, a);
+}
+
 template <bool TOPO>
 void launch_column(const Geo64& G, const ColArgs& a, bool corr, cudaStream_t st) {
-  const unsigned nbc = blocks_for(G.nc, kWarpsPerBlock), nbt = blocks_for(G.nc, 128);
-  if (corr) {
-    k_col_rows_corr<TOPO><<<nbc, 256, 0, st>>>(G, a);
-    k_col_thomas<true><<<nbt, 128, 0, st>>>(G, a);
-    k_col_update<TOPO, true><<<nbc, 256, 0, st>>>(G, a);
-  } else {
-    k_col_rows_pred<TOPO><<<nbc, 256, 0, st>>>(G, a);
-    k_col_thomas<false><<<nbt, 128, 0, st>>>(G, a);
-    k_col_update<TOPO, false><<<nbc, 256, 0, st>>>(G, a);
-  }
+  if (corr) launch_column_as<TOPO, true>(G, a, st);
+  else launch_column_as<TOPO, false>(G, a, st);
 }
 
 }  // namespace
@@ -905,6 +964,11 @@ Geo64 state_geo(const icon_state* st) {
   G.adv_w = s.adv_w;
   G.edge_c = reinterpret_cast<const double4*>(s.edge_c);
   G.lap_w = reinterpret_cast<const double4*>(s.lap_w);
+  // by the cells of the global grid, so that a decomposed domain's parts launch the kernels the
+  // single domain does (its promise is the same bits)
+  const double cells = 4.0 * M_PI * kR * kR / st->abar;
+  G.merge_column = cells < kMergeColumnCells + 0.5;
+  G.merge_stencil = cells < kMergeStencilCells + 0.5;
   const TopoDev& T = s.topo;
   if (T.on) {
     G.t_hsn = T.hsn; G.t_bf = T.bf; G.t_wu_e = T.wu_e; G.t_qinv_dz_e = T.qinv_dz_e; G.t_dz_e = T.dz_e;
@@ -941,10 +1005,14 @@ void fp64_step_stage(icon_state* st, double dt, int nsub, bool corr, cudaStream_
   const double* thv_st = corr ? s.thv_s : s.thv;
   const double* ex_st = corr ? s.ex_s : s.ex;
   prof_begin(stream, K_VERTEX);
-  k_vertex<<<nbv, 256, 0, stream>>>(G, vn_st, w_st, s.zeta, s.w_v);
-  prof_end(stream);
-  prof_begin(stream, K_EDGE_VT);
-  k_edge_vt<<<nbe, 256, 0, stream>>>(G, vn_st, s.vt, s.Ke);
+  if (G.merge_stencil) {
+    k_vertex_edge_vt<<<nbv + nbe, 256, 0, stream>>>(G, vn_st, w_st, s.zeta, s.w_v, s.vt, s.Ke, nbv);
+  } else {
+    k_vertex<<<nbv, 256, 0, stream>>>(G, vn_st, w_st, s.zeta, s.w_v);
+    prof_end(stream);
+    prof_begin(stream, K_EDGE_VT);
+    k_edge_vt<<<nbe, 256, 0, stream>>>(G, vn_st, s.vt, s.Ke);
+  }
   prof_end(stream);
   prof_begin(stream, K_CELL_KE);
   k_cell_ke<<<nbc, 256, 0, stream>>>(G, s.Ke, s.Kc);

@@ -48,10 +48,9 @@ __device__ __forceinline__ void add4(double* m, const F4& x, double w) {
 
 // O3 curl (full levels) and the vertex mean of w (half levels)
 template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_vertex(MxGeo G, const float* __restrict__ vn, const float* __restrict__ w,
-                                                   float* __restrict__ zeta, float* __restrict__ w_v) {
-  QUAD_PROLOGUE(LPE, G.nv)
-  const int64_t v = item;
+__device__ __forceinline__ void mx_vertex_quads(const MxGeo& G, const float* __restrict__ vn,
+                                                const float* __restrict__ w, float* __restrict__ zeta,
+                                                float* __restrict__ w_v, int64_t v, int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2, nh = (G.N + 4) >> 2;
   int64_t E[6], C[6];
   float rw[6];
@@ -87,9 +86,8 @@ __global__ void __launch_bounds__(512) k_mx_vertex(MxGeo G, const float* __restr
 
 // O4 vt
 template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_edge_diag(MxGeo G, const float* __restrict__ vn, float* __restrict__ vt) {
-  QUAD_PROLOGUE(LPE, G.ne)
-  const int64_t e = item;
+__device__ __forceinline__ void mx_edge_diag_quads(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ vt,
+                                                   int64_t e, int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2;
   int64_t S[5];
   float W[5];
@@ -103,6 +101,33 @@ __global__ void __launch_bounds__(512) k_mx_edge_diag(MxGeo G, const float* __re
 #pragma unroll
     for (int j = 0; j < 5; ++j) fma4(acc, W[j], ld4(vn + S[j] + 4 * q));
     st4(vt + e * ld + 4 * q, acc);
+  }
+}
+
+template <int LPE>
+__global__ void __launch_bounds__(512) k_mx_vertex(MxGeo G, const float* __restrict__ vn, const float* __restrict__ w,
+                                                   float* __restrict__ zeta, float* __restrict__ w_v) {
+  QUAD_PROLOGUE(LPE, G.nv)
+  mx_vertex_quads<LPE>(G, vn, w, zeta, w_v, item, lane);
+}
+
+template <int LPE>
+__global__ void __launch_bounds__(512) k_mx_edge_diag(MxGeo G, const float* __restrict__ vn, float* __restrict__ vt) {
+  QUAD_PROLOGUE(LPE, G.ne)
+  mx_edge_diag_quads<LPE>(G, vn, vt, item, lane);
+}
+
+// both in one launch, on small grids (neither reads what the other writes; the first nbv blocks
+// take the vertices)
+__global__ void __launch_bounds__(128) k_mx_vertex_edge(MxGeo G, const float* __restrict__ vn,
+                                                        const float* __restrict__ w, float* __restrict__ zeta,
+                                                        float* __restrict__ w_v, float* __restrict__ vt, unsigned nbv) {
+  const int lane = threadIdx.x & 7;
+  const int64_t item = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 3);
+  if (blockIdx.x < nbv) {
+    if (item < G.nv) mx_vertex_quads<8>(G, vn, w, zeta, w_v, item, lane);
+  } else if (item - (int64_t)nbv * 16 < G.ne) {
+    mx_edge_diag_quads<8>(G, vn, vt, item - (int64_t)nbv * 16, lane);
   }
 }
 
