@@ -420,15 +420,21 @@ bool field_ref(const icon_state* st, int id, void** ptr, int* is_f32, int64_t* n
   }
 }
 
-// the device address of pinned (page-locked, mapped) host memory, or NULL for any other
-// pointer; the query allocates nothing
-const void* mapped_host_ptr(const void* p) {
-  cudaPointerAttributes attr;
-  if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return attr.type == cudaMemoryTypeHost ? attr.devicePointer : nullptr;
+// the device address of n values of pinned (page-locked, mapped) host memory, or NULL for any
+// other pointer, for values that are not aligned, and where the last one is not in the same
+// mapping (a buffer registered in part); the queries allocate nothing
+double* mapped_host_ptr(const double* p, size_t n) {
+  auto device_ptr = [](const double* q) -> double* {
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, q) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return attr.type == cudaMemoryTypeHost ? static_cast<double*>(attr.devicePointer) : nullptr;
+  };
+  if (n == 0 || reinterpret_cast<uintptr_t>(p) % alignof(double) != 0) return nullptr;
+  double* d = device_ptr(p);
+  return d && device_ptr(p + n - 1) == d + (n - 1) ? d : nullptr;
 }
 
 // host-order [n][nlev] <-> the device rows of a field: FP64 or FP32 rows of ld
@@ -769,7 +775,7 @@ int icon_state_copy_field(const icon_state* st, int field_id, double* host_dst, 
   // memory through a device buffer and one contiguous transfer
   const int ld = st->grid->vert.ld;
   cudaStream_t stream = current_stream();
-  double* hd = const_cast<double*>(static_cast<const double*>(mapped_host_ptr(host_dst)));
+  double* hd = mapped_host_ptr(host_dst, count);
   DeviceArena tmp;
   tmp.al = st->arena.al;
   double* stage = hd ? hd : tmp.get_n<double>((size_t)n * nlev);
@@ -802,7 +808,7 @@ int icon_state_set_field(icon_state* st, int field_id, const double* host_src, s
   // pinned memory: the kernel's own reads over the link reach 108 GB/s, the transfer 207)
   const int ld = st->grid->vert.ld;
   cudaStream_t stream = current_stream();
-  double* hs = lm ? nullptr : const_cast<double*>(static_cast<const double*>(mapped_host_ptr(host_src)));
+  double* hs = lm ? nullptr : mapped_host_ptr(host_src, count);
   DeviceArena tmp;
   tmp.al = st->arena.al;
   double* stage = hs ? hs : tmp.get_n<double>((size_t)n * nlev);
@@ -950,6 +956,23 @@ static int tracer_copy(icon_state* st, int t, double* host, size_t count, bool t
   }
   double* dev = st->s.q + (size_t)t * nc * ld;
   cudaStream_t stream = current_stream();
+  // through a packed device buffer and one contiguous transfer (or the pinned buffer itself): a
+  // strided copy of 480-byte rows to pageable memory took 20 ms per tracer at R2B5 / 60 levels
+  // (39 MB). Row by row only where the buffer does not fit
+  double* hp = mapped_host_ptr(host, count);
+  DeviceArena tmp;
+  tmp.al = st->arena.al;
+  if (double* stage = hp ? hp : tmp.get_n<double>(count)) {
+    cudaError_t e = cudaSuccess;
+    if (!to_host && !hp) e = cudaMemcpyAsync(stage, host, sizeof(double) * count, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = move_field(dev, stage, nc, N, ld, false, false, to_host, stream);
+    if (e == cudaSuccess && to_host && !hp)
+      e = cudaMemcpyAsync(host, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    tmp.release();
+    if (e != cudaSuccess) return cuda_fail(e, fn);
+    return ICON_OK;
+  }
   cudaError_t e = to_host ? cudaMemcpy2DAsync(host, sizeof(double) * N, dev, sizeof(double) * ld, sizeof(double) * N,
                                               nc, cudaMemcpyDeviceToHost, stream)
                           : cudaMemcpy2DAsync(dev, sizeof(double) * ld, host, sizeof(double) * N, sizeof(double) * N,
