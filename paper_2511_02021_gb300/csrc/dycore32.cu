@@ -61,74 +61,6 @@ struct MxGeo {
   const float *inv_dz32, *wu32, *wl32, *inv_dz2_32;
 };
 
-// ---------------------------------------------------------------- stencil items (lanes over levels)
-
-// O3 curl (full levels) and the vertex mean of w (half levels)
-template <int LPE>
-__device__ inline void mx_vertex_item(const MxGeo& G, const float* __restrict__ vn, const float* __restrict__ w,
-                                      float* __restrict__ zeta, float* __restrict__ w_v, int64_t v, int lane) {
-  const int ld = G.ld;
-  int64_t E[6], C[6];
-  float rw[6];
-  for (int j = 0; j < 6; ++j) {
-    E[j] = (int64_t)G.v2e[6 * v + j] * ld;
-    C[j] = (int64_t)G.v2c[6 * v + j] * ld;
-    rw[j] = G.rot_w32[6 * v + j];
-  }
-  const int deg = G.vdeg[v];
-  const float inv_deg = 1.0f / (float)deg;
-  for (int k = lane; k < G.N; k += LPE) {
-    float acc = 0.f;
-    for (int j = 0; j < 6; ++j) acc += rw[j] * vn[E[j] + k];
-    zeta[v * ld + k] = acc;
-  }
-  for (int h = lane; h <= G.N; h += LPE) {
-    float acc = 0.f;
-    for (int j = 0; j < 5; ++j) acc += w[C[j] + h];
-    if (deg == 6) acc += w[C[5] + h];
-    w_v[v * ld + h] = acc * inv_deg;
-  }
-}
-
-// O4 vt
-template <int LPE>
-__device__ inline void mx_edge_diag_item(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ vt,
-                                         int64_t e, int lane) {
-  const int ld = G.ld;
-  int64_t S[5];
-  float W[5];
-  for (int j = 0; j < 5; ++j) {
-    S[j] = (int64_t)G.e2vt[5 * e + j] * ld;
-    W[j] = G.vt_w32[5 * e + j];
-  }
-  for (int k = lane; k < G.N; k += LPE) {
-    float acc = 0.f;
-    for (int j = 0; j < 5; ++j) acc += W[j] * vn[S[j] + k];
-    vt[e * ld + k] = acc;
-  }
-}
-
-// O5 K_c = sum_e kappa_ce (vn_e^2 + vt_e^2)/2
-template <int LPE>
-__device__ inline void mx_cell_ke_item(const MxGeo& G, const float* __restrict__ vn, const float* __restrict__ vt,
-                                       float* __restrict__ Kc, int64_t c, int lane) {
-  const int ld = G.ld;
-  int64_t E[3];
-  float kw[3];
-  for (int s = 0; s < 3; ++s) {
-    E[s] = (int64_t)G.c2e[3 * c + s] * ld;
-    kw[s] = G.kin_w32[3 * c + s];
-  }
-  for (int k = lane; k < G.N; k += LPE) {
-    float acc = 0.f;
-    for (int s = 0; s < 3; ++s) {
-      const float a = vn[E[s] + k], b = vt[E[s] + k];
-      acc += kw[s] * (0.5f * (a * a + b * b));
-    }
-    Kc[c * ld + k] = acc;
-  }
-}
-
 struct MxEdgeArgs {
   const float *vn, *w, *rho, *thv, *exp;   // stage state (FP32 shadows; exp = Exner - Exner_ref)
   const float *vt, *Kc, *zeta, *w_v;
@@ -148,112 +80,9 @@ struct MxEdgeArgs {
   const float *t_wu_e, *t_inv_dz_e, *t_dz_e, *t_csn, *t_bf, *t_wcon, *t_hdpdz;
 };
 
-// vn tendency and update, horizontal flux integrals, edge part of the w advection.
-// One pass over the half levels in windows of LPE - 1: lane l of an entity's lane
-// group holds half level h = base + l and, except the last lane, full level k = h;
-// each half-level interpolant and cell-pair sum of w is formed once and passed to the
-// lane below with a shuffle (only the group's own lanes take part, so the two halves
-// of a warp may serve different entities).
-// The persistent ensemble's form: it keeps its arguments in its shared-memory slot and reads
-// them there, which its 64-register budget takes better than holding them (hoisted, its edge
-// phase spilled and slowed from 55 to 79 ms per step).
-template <int LPE>
-__device__ inline void mx_edge_tend_item(const MxGeo& G, const MxEdgeArgs& a, int64_t e, int lane) {
-  const int ld = G.ld, N = G.N;
-  const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
-  const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
-  const float ide = G.inv_de32[e], ile = G.inv_le32[e], fe = G.f_e32[e], le = G.l_e32[e];
-  const float cide = (float)kCpd * ide;
-  const int64_t o = e * ld;
-  const float* __restrict__ vn = a.vn + o;
-  const float* __restrict__ vt = a.vt + o;
-  const float* __restrict__ w = a.w;
-  const float* __restrict__ wv = a.w_v;
-  const float* __restrict__ zeta = a.zeta;
-  const float* __restrict__ Kc = a.Kc;
-  const float* __restrict__ thv = a.thv;
-  const float* __restrict__ exq = a.exp;
-  const float* __restrict__ rho = a.rho;
-  static_assert(LPE == 8 || LPE == 16 || LPE == 32, "lane groups of 8, 16 or 32");
-  const unsigned seg = LPE == 32 ? 0xffffffffu : (((1u << LPE) - 1u) << (threadIdx.x & (32 - LPE)));
-#pragma unroll 2   // two windows' loads in flight (the kernel is bound by load latency)
-  for (int base = 0; base <= N; base += LPE - 1) {
-    const int h = base + lane;
-    const bool hv = h <= N;
-    const int hl = h > 0 ? (h - 1 < N - 1 ? h - 1 : N - 1) : 0;
-    const int hu = h < N ? h : N - 1;
-    const bool inner = h > 0 && h < N;
-    const float wa = inner ? G.wu32[h] : (h == 0 ? 0.0f : 1.0f);
-    const float wb = inner ? G.wl32[h] : (h == 0 ? 1.0f : 0.0f);
-    float vie = 0.f, tie = 0.f, sw = 0.f, dw = 0.f, dwv = 0.f;
-    if (hv) {
-      vie = wa * vn[hl] + wb * vn[hu];
-      tie = wa * vt[hl] + wb * vt[hu];
-      const float w1 = w[c1 + h], w2 = w[c2 + h];
-      sw = w1 + w2;
-      dw = w2 - w1;
-      dwv = wv[v2 + h] - wv[v1 + h];
-    }
-    const float vie_up = __shfl_down_sync(seg, vie, 1, LPE);
-    const float sw_up = __shfl_down_sync(seg, sw, 1, LPE);
-    if (!hv || lane == LPE - 1) continue;
-    a.a_e[o + h] = vie * dw * ide + tie * dwv * ile;
-    if (h == N) continue;
-    const int k = h;
-    const float wbar = 0.25f * (sw + sw_up);
-    const float zeta_e = 0.5f * (zeta[v1 + k] + zeta[v2 + k]);
-    const float A = -(Kc[c2 + k] - Kc[c1 + k]) * ide + (zeta_e + fe) * vt[k] -
-                    wbar * (vie - vie_up) * G.inv_dz32[k];
-    const float t1 = thv[c1 + k], t2 = thv[c2 + k];
-    const float th_e = 0.5f * (t1 + t2);
-    const float pg = th_e * ((exq[c2 + k] - exq[c1 + k]) * cide);
-    float vnew;
-    if (a.corrector) {
-      vnew = a.vn_base[o + k] + a.dtau * (0.5f * (a.Avn0[o + k] + A) - pg);
-    } else {
-      vnew = a.vn_base[o + k] + a.dtau * (A - pg);
-      a.Avn0[o + k] = A;
-    }
-    a.vn_out[o + k] = vnew;
-    if (a.skip_flux) continue;
-    const float F = 0.5f * (rho[c1 + k] + rho[c2 + k]) * vnew;
-    a.phi[o + k] = F;
-    a.gth[o + k] = (le * F) * (a.upwind_theta ? (vnew >= 0.0f ? t1 : t2) : th_e);
-    if (a.corrector) a.mflx[o + k] += f32_to_f64(F) * a.inv_nsub;
-  }
-}
-
 // fourth-order divergence damping of the corrector's vn^{n+1} (option), FP32 like the other
-// stencils: cell divergence, its cell Laplacian, then the edge update with the corrector's
-// fluxes (the same expressions as the edge tendency) and the FP64 step-mean mass flux
-__device__ inline void mx_dd_div_item(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ D, int64_t c,
-                                      int lane) {
-  const int ld = G.ld;
-  int64_t E[3];
-  float dw[3];
-  for (int s = 0; s < 3; ++s) {
-    E[s] = (int64_t)G.c2e[3 * c + s] * ld;
-    dw[s] = G.div_w32[3 * c + s];
-  }
-  for (int k = lane; k < G.N; k += 32) D[c * ld + k] = dw[0] * vn[E[0] + k] + dw[1] * vn[E[1] + k] + dw[2] * vn[E[2] + k];
-}
-
-__device__ inline void mx_dd_lap_item(const MxGeo& G, const float* __restrict__ D, float* __restrict__ L, int64_t c,
-                                      int lane) {
-  const int ld = G.ld;
-  int64_t A[3], B[3];
-  float wt[3];
-  for (int s = 0; s < 3; ++s) {
-    const int e = G.c2e[3 * c + s];
-    A[s] = (int64_t)G.e2c[2 * e] * ld;
-    B[s] = (int64_t)G.e2c[2 * e + 1] * ld;
-    wt[s] = G.div_w32[3 * c + s] * G.inv_de32[e];
-  }
-  for (int k = lane; k < G.N; k += 32)
-    L[c * ld + k] = wt[0] * (D[B[0] + k] - D[A[0] + k]) + wt[1] * (D[B[1] + k] - D[A[1] + k]) +
-                    wt[2] * (D[B[2] + k] - D[A[2] + k]);
-}
-
+// stencils: the edge update with the corrector's fluxes (the same expressions as the edge
+// tendency) and the FP64 step-mean mass flux
 struct MxDDArgs {
   const float *L, *rho, *thv;
   const float* dz_e;                       // layer thickness at edges (terrain-following), or NULL
@@ -277,77 +106,6 @@ __device__ inline void mx_dd_edge_item(const MxGeo& G, const MxDDArgs& a, int64_
     const float t1 = a.thv[c1 + k], t2 = a.thv[c2 + k];
     a.gth[o + k] = (le * F) * (a.upwind_theta ? (vn >= 0.0f ? t1 : t2) : 0.5f * (t1 + t2));
     a.mflx[o + k] += f32_to_f64(F) * a.inv_nsub;
-  }
-}
-
-// diffusion: least-squares vertex velocity and O3 curl of vn
-template <int LPE>
-__device__ inline void mx_diff_vertex_item(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ ux,
-                                           float* __restrict__ uy, float* __restrict__ uz, float* __restrict__ zeta,
-                                           int64_t v, int lane) {
-  const int ld = G.ld;
-  int64_t E[6];
-  for (int j = 0; j < 6; ++j) E[j] = (int64_t)G.v2e[6 * v + j] * ld;
-  const float* lw = G.lsq_w32 + 18 * v;
-  const float* rw = G.rot_w32 + 6 * v;
-  float L[18], R[6];
-  for (int j = 0; j < 18; ++j) L[j] = lw[j];
-  for (int j = 0; j < 6; ++j) R[j] = rw[j];
-  for (int k = lane; k < G.N; k += LPE) {
-    float x = 0.f, y = 0.f, z = 0.f, r = 0.f;
-    for (int j = 0; j < 6; ++j) {
-      const float q = vn[E[j] + k];
-      x += L[3 * j] * q;
-      y += L[3 * j + 1] * q;
-      z += L[3 * j + 2] * q;
-      r += R[j] * q;
-    }
-    ux[v * ld + k] = x;
-    uy[v * ld + k] = y;
-    uz[v * ld + k] = z;
-    zeta[v * ld + k] = r;
-  }
-}
-
-// diffusion: O2 divergence of vn
-template <int LPE>
-__device__ inline void mx_diff_div_item(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ divc,
-                                        int64_t c, int lane) {
-  const int ld = G.ld;
-  int64_t E[3];
-  float dw[3];
-  for (int s = 0; s < 3; ++s) {
-    E[s] = (int64_t)G.c2e[3 * c + s] * ld;
-    dw[s] = G.div_w32[3 * c + s];
-  }
-  for (int k = lane; k < G.N; k += LPE) divc[c * ld + k] = dw[0] * vn[E[0] + k] + dw[1] * vn[E[1] + k] + dw[2] * vn[E[2] + k];
-}
-
-// diffusion: Smagorinsky K_h, vn += dt K_h L(vn), theta_v flux
-template <int LPE>
-__device__ inline void mx_diff_edge_item(const MxGeo& G, float* __restrict__ vn, const float* __restrict__ ux,
-                                         const float* __restrict__ uy, const float* __restrict__ uz,
-                                         const float* __restrict__ zeta, const float* __restrict__ divc,
-                                         const float* __restrict__ thv, float* __restrict__ thflx, float dt, int64_t e,
-                                         int lane) {
-  const int ld = G.ld;
-  int64_t Q[4];
-  for (int j = 0; j < 4; ++j) Q[j] = (int64_t)G.e2q[4 * e + j] * ld;
-  const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
-  const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
-  const float nx = G.n_e32[3 * e], ny = G.n_e32[3 * e + 1], nz = G.n_e32[3 * e + 2];
-  const float tx = G.t_e32[3 * e], ty = G.t_e32[3 * e + 1], tz = G.t_e32[3 * e + 2];
-  const float ide = G.inv_de32[e], ile = G.inv_le32[e], i34 = G.L34inv32[e], le = G.l_e32[e];
-  const float cs2ld = (float)(kCsSmag * kCsSmag) * le / ide;
-  for (int k = lane; k < G.N; k += LPE) {
-    const float ax = ux[Q[3] + k] - ux[Q[2] + k], ay = uy[Q[3] + k] - uy[Q[2] + k], az = uz[Q[3] + k] - uz[Q[2] + k];
-    const float bx = ux[Q[1] + k] - ux[Q[0] + k], by = uy[Q[1] + k] - uy[Q[0] + k], bz = uz[Q[1] + k] - uz[Q[0] + k];
-    const float DT = (ax * nx + ay * ny + az * nz) * i34 - (bx * tx + by * ty + bz * tz) * ile;
-    const float DS = (ax * tx + ay * ty + az * tz) * i34 + (bx * nx + by * ny + bz * nz) * ile;
-    const float Kh = cs2ld * sqrtf(DT * DT + DS * DS);
-    const float lap = (divc[c2 + k] - divc[c1 + k]) * ide - (zeta[v2 + k] - zeta[v1 + k]) * ile;
-    vn[e * ld + k] = vn[e * ld + k] + dt * Kh * lap;
-    thflx[e * ld + k] = le * Kh * (thv[c2 + k] - thv[c1 + k]) * ide;
   }
 }
 
@@ -383,7 +141,15 @@ __global__ void __launch_bounds__(256) k_mx_bd_curldiv(MxGeo G, const float* __r
       zeta1[v * ld + k] = r;
     }
   } else if (item < G.nv + G.nc) {
-    mx_diff_div_item<32>(G, L1, D1, item - G.nv, lane);
+    const int64_t c = item - G.nv;
+    int64_t E[3];
+    float dw[3];
+    for (int s = 0; s < 3; ++s) {
+      E[s] = (int64_t)G.c2e[3 * c + s] * ld;
+      dw[s] = G.div_w32[3 * c + s];
+    }
+    for (int k = lane; k < G.N; k += 32)
+      D1[c * ld + k] = dw[0] * L1[E[0] + k] + dw[1] * L1[E[1] + k] + dw[2] * L1[E[2] + k];
   }
 }
 
@@ -2183,36 +1949,25 @@ __device__ inline void warp_items(const int64_t* off, int nm, int64_t tot, int64
   }
 }
 
-// the same work list taken two items at a time: when both items of a pair belong to one
-// member, the two half-warps take one each with 16 lanes over the levels (f16(m, first item
-// of the pair)); a pair that straddles a member boundary is taken by the whole warp, one
-// item after the other (f32(m, item))
-template <int K, typename F16, typename F32>
-__device__ inline void warp_pairs(const int64_t* off, int nm, int64_t tot, int64_t gwarp, int64_t nwarps, F16 f16,
+// the same work list for the stencils by quads of levels: the warp's four lane groups of eight
+// take an item each (f8(m, first item)); a chunk that straddles a member boundary or the end is
+// taken item by item by the whole warp (f32(m, item))
+template <typename F8, typename F32>
+__device__ inline void warp_quads(const int64_t* off, int nm, int64_t tot, int64_t gwarp, int64_t nwarps, F8 f8,
                                   F32 f32) {
-  static_assert(K % 2 == 0, "pairs");
-  for (int64_t i0 = gwarp * K; i0 < tot; i0 += nwarps * K) {
+  for (int64_t i0 = gwarp * 4; i0 < tot; i0 += nwarps * 4) {
     int m = find_member(off, nm, i0);
     int64_t next = m + 1 < nm ? off[m + 1] : tot;
-    for (int j = 0; j < K; j += 2) {
-      const int64_t i = i0 + j;
-      if (i >= tot) break;
+    if (i0 + 4 <= next) {
+      f8(m, i0 - off[m]);
+      continue;
+    }
+    for (int64_t i = i0; i < i0 + 4 && i < tot; ++i) {
       while (i >= next) {
         ++m;
         next = m + 1 < nm ? off[m + 1] : tot;
       }
-      if (i + 1 < next) {
-        f16(m, i - off[m]);
-      } else {
-        f32(m, i - off[m]);
-        if (i + 1 < tot) {
-          while (i + 1 >= next) {
-            ++m;
-            next = m + 1 < nm ? off[m + 1] : tot;
-          }
-          f32(m, i + 1 - off[m]);
-        }
-      }
+      f32(m, i - off[m]);
     }
   }
 }
@@ -2378,61 +2133,77 @@ __global__ void __launch_bounds__(128, MINB) k_ensemble_step(EnsArgs A) {
   if (!sync(ICON_ENS_PH_ZERO)) return;
   for (int it = 0; it < A.nsub; ++it) {
     for (int stage = 0; stage < 2; ++stage) {
-      // the stencil phases take two entities per warp (16 lanes over the levels each), as
-      // the per-state kernels' tuned tiles do
-      warp_pairs<kChunk>(
+      // the stencil phases take four entities per warp, four levels per lane, as the per-state
+      // kernels do (32 states of R2B4/60 and 32 of R2B5/60, per step: vertices 9.2 -> 7.0 ms, edge
+      // diagnostics 11.2 -> 7.2, kinetic energy 9.4 -> 6.2, edge tendency 54.1 -> 42.2, damping
+      // 10.3 -> 5.3, diffusion 13.7 -> 12.6). The edge tendency is still the slower for the 64
+      // registers that eight blocks per SM leave it (85 registers: 34.5 ms, but the column 79.0
+      // -> 83.4 and the gather 51.8 -> 57.0, the step 211.6 -> 216.5)
+      warp_quads(
           s_off_v, A.nm, A.tot_v, gwarp, nwarps,
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_vertex_item<16>(geo(m), M.ea[stage].vn, M.ea[stage].w, M.zeta32, M.wv32, j + (lane >> 4), lane & 15);
+            mx_vertex_quads<8>(geo(m), M.ea[stage].vn, M.ea[stage].w, M.zeta32, M.wv32, j + (lane >> 3), lane & 7);
           },
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_vertex_item<32>(geo(m), M.ea[stage].vn, M.ea[stage].w, M.zeta32, M.wv32, j, lane);
+            mx_vertex_quads<32>(geo(m), M.ea[stage].vn, M.ea[stage].w, M.zeta32, M.wv32, j, lane);
           });
       if (!sync(ICON_ENS_PH_VERTEX)) return;
-      warp_pairs<kChunk>(
+      warp_quads(
           s_off_e, A.nm, A.tot_e, gwarp, nwarps,
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_edge_diag_item<16>(geo(m), M.ea[stage].vn, M.vt32, j + (lane >> 4), lane & 15);
+            mx_edge_diag_quads<8>(geo(m), M.ea[stage].vn, M.vt32, j + (lane >> 3), lane & 7);
           },
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_edge_diag_item<32>(geo(m), M.ea[stage].vn, M.vt32, j, lane);
+            mx_edge_diag_quads<32>(geo(m), M.ea[stage].vn, M.vt32, j, lane);
           });
       if (!sync(ICON_ENS_PH_EDGE_DIAG)) return;
-      warp_pairs<kChunk>(
+      warp_quads(
           s_off_c, A.nm, A.tot_c, gwarp, nwarps,
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_cell_ke_item<16>(geo(m), M.ea[stage].vn, M.vt32, M.Kc32, j + (lane >> 4), lane & 15);
+            mx_cell_ke_quads<8>(geo(m), M.ea[stage].vn, M.vt32, M.Kc32, j + (lane >> 3), lane & 7);
           },
           [&](int m, int64_t j) {
             const MemberDev& M = A.m[m];
-            mx_cell_ke_item<32>(geo(m), M.ea[stage].vn, M.vt32, M.Kc32, j, lane);
+            mx_cell_ke_quads<32>(geo(m), M.ea[stage].vn, M.vt32, M.Kc32, j, lane);
           });
       if (!sync(ICON_ENS_PH_CELL_KE)) return;
       arg_m = -1;
-      warp_pairs<kChunk>(
+      warp_quads(
           s_off_e, A.nm, A.tot_e, gwarp, nwarps,
           [&](int m, int64_t j) {
-            mx_edge_tend_item<16>(geo(m), edge_args_of(m, stage), j + (lane >> 4), lane & 15);
+            mx_edge_tend_quads<8, false, true>(geo(m), edge_args_of(m, stage), j + (lane >> 3), lane & 7);
           },
-          [&](int m, int64_t j) { mx_edge_tend_item<32>(geo(m), edge_args_of(m, stage), j, lane); });
+          [&](int m, int64_t j) { mx_edge_tend_quads<32, false, true>(geo(m), edge_args_of(m, stage), j, lane); });
       if (!sync(ICON_ENS_PH_EDGE_TEND)) return;
       if (stage == 1 && A.any_damp) {
         // divergence damping of vn^{n+1}: cell divergence (into Kc32), its Laplacian (into
         // vt32), then the edge update with the fluxes the edge tendency left out
-        warp_items<kChunk>(s_off_c, A.nm, A.tot_c, gwarp, nwarps, [&](int m, int64_t j) {
-          const MemberDev& M = A.m[m];
-          if (M.damp) mx_dd_div_item(geo(m), M.dd.vn, M.Kc32, j, lane);
-        });
+        warp_quads(
+            s_off_c, A.nm, A.tot_c, gwarp, nwarps,
+            [&](int m, int64_t j) {
+              const MemberDev& M = A.m[m];
+              if (M.damp) mx_div_quads<8>(geo(m), M.dd.vn, M.Kc32, j + (lane >> 3), lane & 7);
+            },
+            [&](int m, int64_t j) {
+              const MemberDev& M = A.m[m];
+              if (M.damp) mx_div_quads<32>(geo(m), M.dd.vn, M.Kc32, j, lane);
+            });
         if (!sync(ICON_ENS_PH_DD_DIV)) return;
-        warp_items<kChunk>(s_off_c, A.nm, A.tot_c, gwarp, nwarps, [&](int m, int64_t j) {
-          const MemberDev& M = A.m[m];
-          if (M.damp) mx_dd_lap_item(geo(m), M.Kc32, M.vt32, j, lane);
-        });
+        warp_quads(
+            s_off_c, A.nm, A.tot_c, gwarp, nwarps,
+            [&](int m, int64_t j) {
+              const MemberDev& M = A.m[m];
+              if (M.damp) mx_dd_lap_quads<8>(geo(m), M.Kc32, M.vt32, j + (lane >> 3), lane & 7);
+            },
+            [&](int m, int64_t j) {
+              const MemberDev& M = A.m[m];
+              if (M.damp) mx_dd_lap_quads<32>(geo(m), M.Kc32, M.vt32, j, lane);
+            });
         if (!sync(ICON_ENS_PH_DD_LAP)) return;
         if (!LEAN) {     // the lean column's gather forms the damped fluxes itself
           warp_items<kChunk>(s_off_e, A.nm, A.tot_e, gwarp, nwarps, [&](int m, int64_t j) {
@@ -2503,24 +2274,39 @@ __global__ void __launch_bounds__(128, MINB) k_ensemble_step(EnsArgs A) {
     }
   }
   // diffusion
-  for (int64_t i = gwarp; i < A.tot_v + A.tot_c; i += nwarps) {
-    if (i < A.tot_v) {
-      const int m = find_member(s_off_v, A.nm, i);
-      const MemberDev& M = A.m[m];
-      mx_diff_vertex_item<32>(M.G, M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, i - M.off_v, lane);
-    } else {
-      const int64_t j = i - A.tot_v;
-      const int m = find_member(s_off_c, A.nm, j);
-      const MemberDev& M = A.m[m];
-      mx_diff_div_item<32>(M.G, M.vn32, M.Kc32, j - M.off_c, lane);
-    }
-  }
+  warp_quads(
+      s_off_v, A.nm, A.tot_v, gwarp, nwarps,
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_diff_vertex_quads<8>(geo(m), M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, j + (lane >> 3), lane & 7);
+      },
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_diff_vertex_quads<32>(geo(m), M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, j, lane);
+      });
+  warp_quads(
+      s_off_c, A.nm, A.tot_c, gwarp, nwarps,
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_div_quads<8>(geo(m), M.vn32, M.Kc32, j + (lane >> 3), lane & 7);
+      },
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_div_quads<32>(geo(m), M.vn32, M.Kc32, j, lane);
+      });
   if (!sync(ICON_ENS_PH_DIFF_VERTEX)) return;
-  warp_items<kChunk>(s_off_e, A.nm, A.tot_e, gwarp, nwarps, [&](int m, int64_t j) {
-    const MemberDev& M = A.m[m];
-    mx_diff_edge_item<32>(M.G, M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, M.Kc32, M.thv32, M.vt32, (float)M.dt,
-                          j, lane);
-  });
+  warp_quads(
+      s_off_e, A.nm, A.tot_e, gwarp, nwarps,
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_diff_edge_quads<8>(geo(m), M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, M.Kc32, M.thv32, M.vt32,
+                              (float)M.dt, nullptr, nullptr, 0.0f, j + (lane >> 3), lane & 7);
+      },
+      [&](int m, int64_t j) {
+        const MemberDev& M = A.m[m];
+        mx_diff_edge_quads<32>(geo(m), M.vn32, M.uvx32, M.uvy32, M.uvz32, M.zeta32, M.Kc32, M.thv32, M.vt32,
+                              (float)M.dt, nullptr, nullptr, 0.0f, j, lane);
+      });
   if (!sync(ICON_ENS_PH_DIFF_EDGE)) return;
   for (int64_t i = gtid; i < A.tot_c; i += nthreads) {
     const int m = find_member(s_off_c, A.nm, i);

@@ -133,10 +133,9 @@ __global__ void __launch_bounds__(128) k_mx_vertex_edge(MxGeo G, const float* __
 
 // O5 K_c = sum_e kappa_ce (vn_e^2 + vt_e^2)/2
 template <int LPE>
-__global__ void __launch_bounds__(512) k_mx_cell_ke(MxGeo G, const float* __restrict__ vn, const float* __restrict__ vt,
-                                                    float* __restrict__ Kc) {
-  QUAD_PROLOGUE(LPE, G.nc)
-  const int64_t c = item;
+__device__ __forceinline__ void mx_cell_ke_quads(const MxGeo& G, const float* __restrict__ vn,
+                                                 const float* __restrict__ vt, float* __restrict__ Kc, int64_t c,
+                                                 int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2;
   int64_t E[3];
   float kw[3];
@@ -158,17 +157,23 @@ __global__ void __launch_bounds__(512) k_mx_cell_ke(MxGeo G, const float* __rest
   }
 }
 
+template <int LPE>
+__global__ void __launch_bounds__(512) k_mx_cell_ke(MxGeo G, const float* __restrict__ vn, const float* __restrict__ vt,
+                                                    float* __restrict__ Kc) {
+  QUAD_PROLOGUE(LPE, G.nc)
+  mx_cell_ke_quads<LPE>(G, vn, vt, Kc, item, lane);
+}
+
 // vn tendency and update, horizontal flux integrals, edge part of the w advection. A lane holds
 // the half levels of its quad and the one below it (five: the interpolants the quad's full levels
 // difference; the fifth is formed again by the next lane rather than shuffled). Where a sum has
 // two products, the one rounded first is written out, as the one-level form had it. TOPO
 // (terrain-following levels): per-edge interpolation weights, w - wcc in the vertical advection,
 // the metric correction of the pressure gradient (exp is then against the per-cell reference),
-// fluxes through dz_e.
-template <int LPE, bool TOPO>
-__global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
-  QUAD_PROLOGUE(LPE, G.ne)
-  const int64_t e = item;
+// fluxes through dz_e. ROUND_PG: the predictor subtracts the rounded pressure gradient instead of
+// fusing the product (the persistent ensemble's results are defined so).
+template <int LPE, bool TOPO, bool ROUND_PG = false>
+__device__ __forceinline__ void mx_edge_tend_quads(const MxGeo& G, const MxEdgeArgs& a, int64_t e, int lane) {
   const int ld = G.ld, N = G.N, nh = (N + 4) >> 2;
   const int64_t c1 = (int64_t)G.e2c[2 * e] * ld, c2 = (int64_t)G.e2c[2 * e + 1] * ld;
   const int64_t v1 = (int64_t)G.e2v[2 * e] * ld, v2 = (int64_t)G.e2v[2 * e + 1] * ld;
@@ -260,7 +265,8 @@ __global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) 
       else px = __fmul_rn(p2.v[i] - p1.v[i], cide);
       if (corr)
         vo.v[i] = __fmaf_rn(dtau, __fmaf_rn(0.5f, av.v[i] + A.v[i], -__fmul_rn(th_e, px)), vb.v[i]);
-      else vo.v[i] = __fmaf_rn(dtau, __fmaf_rn(-th_e, px, A.v[i]), vb.v[i]);
+      else
+        vo.v[i] = __fmaf_rn(dtau, ROUND_PG ? __fsub_rn(A.v[i], __fmul_rn(th_e, px)) : __fmaf_rn(-th_e, px, A.v[i]), vb.v[i]);
     }
     if (!corr) st4(avn_o + k0, A);
     st4(vout_o + k0, vo);
@@ -280,13 +286,19 @@ __global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) 
   }
 }
 
+template <int LPE, bool TOPO>
+__global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
+  QUAD_PROLOGUE(LPE, G.ne)
+  mx_edge_tend_quads<LPE, TOPO>(G, a, item, lane);
+}
+
 // ---- fourth-order divergence damping of the corrector's vn^{n+1}: cell divergence, its cell
 // Laplacian, then the edge update (eight lanes per entity, four entities per warp)
 constexpr int kQuadLanes = 8;
 
-__global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restrict__ vn, float* __restrict__ D) {
-  QUAD_PROLOGUE(kQuadLanes, G.nc)
-  const int64_t c = item;
+template <int LPE>
+__device__ __forceinline__ void mx_div_quads(const MxGeo& G, const float* __restrict__ vn, float* __restrict__ D,
+                                             int64_t c, int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2;
   int64_t E[3];
   float dw[3];
@@ -295,7 +307,7 @@ __global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restr
     E[s] = (int64_t)G.c2e[3 * c + s] * ld;
     dw[s] = G.div_w32[3 * c + s];
   }
-  for (int q = lane; q < nq; q += kQuadLanes) {
+  for (int q = lane; q < nq; q += LPE) {
     const F4 x0 = ld4(vn + E[0] + 4 * q), x1 = ld4(vn + E[1] + 4 * q), x2 = ld4(vn + E[2] + 4 * q);
     F4 d;
 #pragma unroll
@@ -304,9 +316,14 @@ __global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restr
   }
 }
 
-__global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restrict__ D, float* __restrict__ L) {
+__global__ void __launch_bounds__(256) k_mx_dd_div(MxGeo G, const float* __restrict__ vn, float* __restrict__ D) {
   QUAD_PROLOGUE(kQuadLanes, G.nc)
-  const int64_t c = item;
+  mx_div_quads<kQuadLanes>(G, vn, D, item, lane);
+}
+
+template <int LPE>
+__device__ __forceinline__ void mx_dd_lap_quads(const MxGeo& G, const float* __restrict__ D, float* __restrict__ L,
+                                                int64_t c, int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2;
   int64_t B[3];
   float wt[3];
@@ -319,7 +336,7 @@ __global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restr
     B[s] = (int64_t)(out[s] ? cb : ca) * ld;
     wt[s] = G.div_w32[3 * c + s] * G.inv_de32[e];
   }
-  for (int q = lane; q < nq; q += kQuadLanes) {
+  for (int q = lane; q < nq; q += LPE) {
     const F4 m = ld4(D + c * ld + 4 * q);                    // own row once, not once per edge
     const F4 x0 = ld4(D + B[0] + 4 * q), x1 = ld4(D + B[1] + 4 * q), x2 = ld4(D + B[2] + 4 * q);
     F4 l;
@@ -332,6 +349,11 @@ __global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restr
     }
     st4(L + c * ld + 4 * q, l);
   }
+}
+
+__global__ void __launch_bounds__(256) k_mx_dd_lap(MxGeo G, const float* __restrict__ D, float* __restrict__ L) {
+  QUAD_PROLOGUE(kQuadLanes, G.nc)
+  mx_dd_lap_quads<kQuadLanes>(G, D, L, item, lane);
 }
 
 // the damping's edge update with the corrector's fluxes and the FP64 step-mean mass flux. A kernel
@@ -365,70 +387,58 @@ __global__ void __launch_bounds__(256, 4) k_mx_dd_edge(MxGeo G, MxDDArgs a) {
   }
 }
 
-// ---- diffusion: least-squares vertex velocity and O3 curl of vn (vertices first), O2
-// divergence (then cells); both only read vn
+// ---- diffusion: least-squares vertex velocity and O3 curl of vn
+template <int LPE>
+__device__ __forceinline__ void mx_diff_vertex_quads(const MxGeo& G, const float* __restrict__ vn,
+                                                     float* __restrict__ ux, float* __restrict__ uy,
+                                                     float* __restrict__ uz, float* __restrict__ zeta, int64_t v,
+                                                     int lane) {
+  const int ld = G.ld, nq = (G.N + 3) >> 2;
+  int64_t E[6];
+  float L[18], R[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) E[j] = (int64_t)G.v2e[6 * v + j] * ld;
+#pragma unroll
+  for (int j = 0; j < 18; ++j) L[j] = G.lsq_w32[18 * v + j];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) R[j] = G.rot_w32[6 * v + j];
+  for (int q = lane; q < nq; q += LPE) {
+    F4 x{}, y{}, z{}, r{};
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const F4 u = ld4(vn + E[j] + 4 * q);
+      fma4(x, L[3 * j], u);
+      fma4(y, L[3 * j + 1], u);
+      fma4(z, L[3 * j + 2], u);
+      fma4(r, R[j], u);
+    }
+    const int64_t o = v * ld + 4 * q;
+    st4(ux + o, x);
+    st4(uy + o, y);
+    st4(uz + o, z);
+    st4(zeta + o, r);
+  }
+}
+
+// vertices first, then O2 divergence at the cells; both only read vn
 template <int LPE>
 __global__ void __launch_bounds__(512, 2) k_mx_diff_vertex(MxGeo G, const float* __restrict__ vn, float* __restrict__ ux,
                                                         float* __restrict__ uy, float* __restrict__ uz,
                                                         float* __restrict__ zeta, float* __restrict__ divc) {
   QUAD_PROLOGUE(LPE, G.nv + G.nc)
-  const int ld = G.ld, nq = (G.N + 3) >> 2;
-  if (item < G.nv) {
-    const int64_t v = item;
-    int64_t E[6];
-    float L[18], R[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) E[j] = (int64_t)G.v2e[6 * v + j] * ld;
-#pragma unroll
-    for (int j = 0; j < 18; ++j) L[j] = G.lsq_w32[18 * v + j];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) R[j] = G.rot_w32[6 * v + j];
-    for (int q = lane; q < nq; q += LPE) {
-      F4 x{}, y{}, z{}, r{};
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        const F4 u = ld4(vn + E[j] + 4 * q);
-        fma4(x, L[3 * j], u);
-        fma4(y, L[3 * j + 1], u);
-        fma4(z, L[3 * j + 2], u);
-        fma4(r, R[j], u);
-      }
-      const int64_t o = v * ld + 4 * q;
-      st4(ux + o, x);
-      st4(uy + o, y);
-      st4(uz + o, z);
-      st4(zeta + o, r);
-    }
-  } else {
-    const int64_t c = item - G.nv;
-    int64_t E[3];
-    float dw[3];
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      E[s] = (int64_t)G.c2e[3 * c + s] * ld;
-      dw[s] = G.div_w32[3 * c + s];
-    }
-    for (int q = lane; q < nq; q += LPE) {
-      const F4 x0 = ld4(vn + E[0] + 4 * q), x1 = ld4(vn + E[1] + 4 * q), x2 = ld4(vn + E[2] + 4 * q);
-      F4 d;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) d.v[i] = dw[0] * x0.v[i] + dw[1] * x1.v[i] + dw[2] * x2.v[i];
-      st4(divc + c * ld + 4 * q, d);
-    }
-  }
+  if (item < G.nv) mx_diff_vertex_quads<LPE>(G, vn, ux, uy, uz, zeta, item, lane);
+  else mx_div_quads<LPE>(G, vn, divc, item - G.nv, lane);
 }
 
 // diffusion: Smagorinsky K_h, vn += dt K_h L(vn), theta_v flux; D1 and zeta1 (fourth-order
 // background diffusion, an option) or NULL
-__global__ void __launch_bounds__(256, 2) k_mx_diff_edge(MxGeo G, float* __restrict__ vn, const float* __restrict__ ux,
-                                                         const float* __restrict__ uy, const float* __restrict__ uz,
-                                                         const float* __restrict__ zeta,
-                                                         const float* __restrict__ divc, const float* __restrict__ thv,
-                                                         float* __restrict__ thflx, float dt,
-                                                         const float* __restrict__ D1, const float* __restrict__ zeta1,
-                                                         float bd_scale) {
-  QUAD_PROLOGUE(kQuadLanes, G.ne)
-  const int64_t e = item;
+template <int LPE>
+__device__ __forceinline__ void mx_diff_edge_quads(const MxGeo& G, float* __restrict__ vn, const float* __restrict__ ux,
+                                                   const float* __restrict__ uy, const float* __restrict__ uz,
+                                                   const float* __restrict__ zeta, const float* __restrict__ divc,
+                                                   const float* __restrict__ thv, float* __restrict__ thflx, float dt,
+                                                   const float* __restrict__ D1, const float* __restrict__ zeta1,
+                                                   float bd_scale, int64_t e, int lane) {
   const int ld = G.ld, nq = (G.N + 3) >> 2;
   int64_t Q[4];
 #pragma unroll
@@ -439,7 +449,7 @@ __global__ void __launch_bounds__(256, 2) k_mx_diff_edge(MxGeo G, float* __restr
   const float tx = G.t_e32[3 * e], ty = G.t_e32[3 * e + 1], tz = G.t_e32[3 * e + 2];
   const float ide = G.inv_de32[e], ile = G.inv_le32[e], i34 = G.L34inv32[e], le = G.l_e32[e];
   const float cs2ld = (float)(kCsSmag * kCsSmag) * le / ide;
-  for (int q = lane; q < nq; q += kQuadLanes) {
+  for (int q = lane; q < nq; q += LPE) {
     const int k = 4 * q;
     const F4 x3 = ld4(ux + Q[3] + k), x2 = ld4(ux + Q[2] + k), x1 = ld4(ux + Q[1] + k), x0 = ld4(ux + Q[0] + k);
     const F4 y3 = ld4(uy + Q[3] + k), y2 = ld4(uy + Q[2] + k), y1 = ld4(uy + Q[1] + k), y0 = ld4(uy + Q[0] + k);
@@ -469,6 +479,17 @@ __global__ void __launch_bounds__(256, 2) k_mx_diff_edge(MxGeo G, float* __restr
     st4(vn + e * ld + k, vo);
     st4(thflx + e * ld + k, fl);
   }
+}
+
+__global__ void __launch_bounds__(256, 2) k_mx_diff_edge(MxGeo G, float* __restrict__ vn, const float* __restrict__ ux,
+                                                         const float* __restrict__ uy, const float* __restrict__ uz,
+                                                         const float* __restrict__ zeta,
+                                                         const float* __restrict__ divc, const float* __restrict__ thv,
+                                                         float* __restrict__ thflx, float dt,
+                                                         const float* __restrict__ D1, const float* __restrict__ zeta1,
+                                                         float bd_scale) {
+  QUAD_PROLOGUE(kQuadLanes, G.ne)
+  mx_diff_edge_quads<kQuadLanes>(G, vn, ux, uy, uz, zeta, divc, thv, thflx, dt, D1, zeta1, bd_scale, item, lane);
 }
 
 // ---- diffusion of theta_v: FP32 increment, FP64 accumulation, Exner at constant density,
