@@ -27,12 +27,12 @@
 //    frozen at S^n. After the FP64 back substitution, the predictor forms those
 //    shadows' implicit increments in FP32.
 //
-// Every kernel body is a per-item device function (one entity for the stencils,
-// one column for the solve) shared by the per-state kernels and by the persistent
-// ensemble kernel. The stencil kernels take the number of lanes per entity (32 or
-// 16: one or two entities per warp) and the block size from the autotuner; each
-// output is computed by one lane with a fixed summation order, so the results do
-// not depend on the tile shape.
+// The stencils (stencils32.h: four levels per lane, a template argument for the lanes
+// per entity) are per-item device functions shared by the per-state kernels and the
+// persistent ensemble kernel. The lean column has per-state kernels of its own
+// (lean_column.h); the ensemble keeps one warp per 32 columns, which fits the registers
+// its other phases leave. Each output is computed by one lane with a fixed summation
+// order, so the results do not depend on the tile shape.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -972,112 +972,6 @@ struct LeanTile {
   float t[4][CH][33];                      // rho, theta_v, pi - pi_ref, w of 32 columns
 };
 
-// gather of the lean column's stage inputs for 32 consecutive cells: lanes over levels
-// (LPE per cell), transposed through shared memory into level-major rows (the persistent ensemble's form)
-template <int LPE>
-struct LeanGatherTile {
-  double d[LPE][kGatherCells + 1];
-  float f[4][LPE][kGatherCells + 1];       // dtau D_Theta, dtau A_w, A_w (predictor), dtau D_rho (predictor)
-};
-
-template <int LPE, bool CORR, bool DDF = false>
-__device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, int64_t c0, LeanGatherTile<LPE>& T) {
-  constexpr int CB = kGatherCells;
-  const int N = G.N, ld = G.ld;
-  const int64_t nc = G.nc;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int grp = tid / LPE, ngrp = nthr / LPE, lane = tid % LPE;
-  const float dtau32 = (float)a.dtau;
-  for (int k0 = 0; k0 < N; k0 += LPE) {
-    if (CORR) {
-      for (int i = tid; i < LPE * CB; i += nthr) {
-        const int r = i / CB, cl = i % CB, h = k0 + r;
-        const int64_t c = c0 + cl;
-        T.f[2][r][cl] = (h >= 1 && h < N && c < nc) ? a.Aw0[(int64_t)h * nc + c] : 0.0f;
-      }
-      __syncthreads();
-    }
-    for (int cl = grp; cl < CB; cl += ngrp) {
-      const int64_t c = c0 + cl;
-      if (c >= nc) break;
-      const int64_t o = c * ld;
-      int64_t E[3];
-      float sg[3], kw[3];
-      double dwt[3];
-      const float4 cw = a.cw32[c];
-      const float dw32[3] = {cw.x, cw.y, cw.z};
-      int64_t Ca[3], Cb[3];                  // DDF: the edges' two cells (row offsets)
-      float sc[3], le[3];
-      bool own[3];
-      for (int s = 0; s < 3; ++s) {
-        const int e = G.c2e[3 * c + s];
-        E[s] = (int64_t)e * ld;
-        sg[s] = G.s_ce32[3 * c + s];
-        kw[s] = G.kin_w32[3 * c + s];
-        if (CORR) dwt[s] = a.dwa_t[3 * c + s];
-        if (DDF) {
-          const int ca = G.e2c[2 * e], cb = G.e2c[2 * e + 1];
-          Ca[s] = (int64_t)ca * ld;
-          Cb[s] = (int64_t)cb * ld;
-          sc[s] = a.dd_scale * G.inv_de32[e];
-          le[s] = G.l_e32[e];
-          own[s] = ca == c;
-        }
-      }
-      const float ta = cw.w;
-      const int k = k0 + lane;
-      if (k < N) {
-        float F[3], Gt[3];
-        if (DDF) {
-          // damped vn^{n+1} and its fluxes, as the damping's edge update forms them
-          for (int s = 0; s < 3; ++s) {
-            const float vd = a.dd_vn[E[s] + k] - sc[s] * (a.dd_L[Cb[s] + k] - a.dd_L[Ca[s] + k]);
-            F[s] = 0.5f * (a.dd_rho[Ca[s] + k] + a.dd_rho[Cb[s] + k]) * vd;
-            const float t1 = a.dd_thv[Ca[s] + k], t2 = a.dd_thv[Cb[s] + k];
-            Gt[s] = (le[s] * F[s]) * (a.dd_upwind ? (vd >= 0.0f ? t1 : t2) : 0.5f * (t1 + t2));
-            if (own[s]) {
-              a.dd_out[E[s] + k] = vd;
-              a.mflx[E[s] + k] += (double)F[s] * a.inv_nsub;
-            }
-          }
-        } else {
-          for (int s = 0; s < 3; ++s) {
-            F[s] = a.phi[E[s] + k];
-            Gt[s] = a.gth[E[s] + k];
-          }
-        }
-        // the hardware conversion here: the gather leaves the FP64 pipe half idle, and the
-        // integer-pipe form costs more issue slots (measured 6.0 against 5.6 ms per step)
-        if (CORR) T.d[lane][cl] = (dwt[0] * (double)F[0] + dwt[1] * (double)F[1]) + dwt[2] * (double)F[2];
-        else T.f[3][lane][cl] = (dw32[0] * F[0] + dw32[1] * F[1]) + dw32[2] * F[2];
-        T.f[0][lane][cl] = (sg[0] * Gt[0] + sg[1] * Gt[1] + sg[2] * Gt[2]) * ta;
-      }
-      if (k >= 1 && k < N) {
-        const float hadv = kw[0] * a.a_e[E[0] + k] + kw[1] * a.a_e[E[1] + k] + kw[2] * a.a_e[E[2] + k];
-        float Aw = -hadv - a.w_stage[o + k] * (a.w_stage[o + k - 1] - a.w_stage[o + k + 1]) * G.inv_dz2_32[k];
-        if (CORR) Aw = 0.5f * (T.f[2][lane][cl] + Aw);
-        else T.f[2][lane][cl] = Aw;
-        T.f[1][lane][cl] = dtau32 * Aw;
-      }
-    }
-    __syncthreads();
-    for (int i = tid; i < LPE * CB; i += nthr) {
-      const int r = i / CB, cl = i % CB, k = k0 + r;
-      const int64_t c = c0 + cl;
-      if (c >= nc || k >= N) continue;
-      const int64_t j = (int64_t)k * nc + c;
-      if (CORR) a.dr64[j] = T.d[r][cl];
-      else a.dr32[j] = T.f[3][r][cl];
-      a.dt32[j] = T.f[0][r][cl];
-      if (k >= 1) {
-        a.aw32[j] = T.f[1][r][cl];
-        if (!CORR) a.Aw0[j] = T.f[2][r][cl];
-      }
-    }
-    __syncthreads();
-  }
-}
-
 // write the finished chunk [k0, k0 + CH) of the warp's 32 columns (first cell c0): CH lanes
 // per column row, 32 / CH rows per store instruction
 template <int CH>
@@ -1320,6 +1214,111 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
 
 #include "stencils32.h"
 #include "lean_column.h"
+
+// gather of the lean column's stage inputs for 32 consecutive cells, the persistent ensemble's
+// form: LPE levels per pass, four per lane in 128-bit loads, transposed through shared memory into
+// level-major rows; the predictor's A_w is averaged in as the rows are written, where it is read
+// coalesced. DDF: the damping's edge update is formed here by both cells of an edge, edge by edge
+// (at four levels per lane one edge's neighbour rows fill the registers that the phase has).
+// 32 states of R2B4/60 and 32 of R2B5/60: 52.7 ms per step with one level per lane, 35.0 now
+template <int LPE>
+struct LeanGatherTile {
+  double d[LPE][kGatherCells + 1];
+  float f[3][LPE][kGatherCells + 1];       // dtau D_Theta, A_w, dtau D_rho (predictor)
+};
+
+template <int LPE, bool CORR, bool DDF = false>
+__device__ inline void mx_lean_gather_body(const MxGeo& G, const MxLeanArgs& a, int64_t c0, LeanGatherTile<LPE>& T) {
+  constexpr int CB = kGatherCells, QL = LPE / 4;     // lanes per cell, four levels each
+  const int N = G.N, ld = G.ld;
+  const int64_t nc = G.nc;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int grp = tid / QL, ngrp = nthr / QL, lane = tid % QL;
+  const float dtau32 = (float)a.dtau;
+  for (int k0 = 0; k0 < N; k0 += LPE) {
+    const int k = k0 + 4 * lane;
+    for (int cl = grp; cl < CB; cl += ngrp) {
+      const int64_t c = c0 + cl;
+      if (c >= nc || k >= N) break;
+      const int64_t o = c * ld;
+      int64_t E[3];
+      F4 F[3], Gt[3];
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        const int e = G.c2e[3 * c + s];
+        E[s] = (int64_t)e * ld;
+        if constexpr (DDF) {
+          // damped vn^{n+1} and its fluxes, as the damping's edge update forms them
+          const int ca = G.e2c[2 * e], cb = G.e2c[2 * e + 1];
+          const int64_t A = (int64_t)ca * ld + k, B = (int64_t)cb * ld + k;
+          const float sc = a.dd_scale * G.inv_de32[e], le = G.l_e32[e];
+          F4 vd = ld4(a.dd_vn + E[s] + k);
+          {
+            const F4 L1 = ld4(a.dd_L + A), L2 = ld4(a.dd_L + B);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) vd.v[i] = __fmaf_rn(-sc, L2.v[i] - L1.v[i], vd.v[i]);
+          }
+          const F4 r1 = ld4(a.dd_rho + A), r2 = ld4(a.dd_rho + B), t1 = ld4(a.dd_thv + A), t2 = ld4(a.dd_thv + B);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            F[s].v[i] = 0.5f * (r1.v[i] + r2.v[i]) * vd.v[i];
+            Gt[s].v[i] = (le * F[s].v[i]) *
+                         (a.dd_upwind ? (vd.v[i] >= 0.0f ? t1.v[i] : t2.v[i]) : 0.5f * (t1.v[i] + t2.v[i]));
+          }
+          if (ca == c) {
+            st4(a.dd_out + E[s] + k, vd);
+            add4(a.mflx + E[s] + k, F[s], a.inv_nsub);
+          }
+        } else {
+          F[s] = ld4(a.phi + E[s] + k);
+          Gt[s] = ld4(a.gth + E[s] + k);
+        }
+      }
+      {
+        const float4 cw = a.cw32[c];
+        const float g0 = G.s_ce32[3 * c], g1 = G.s_ce32[3 * c + 1], g2 = G.s_ce32[3 * c + 2];
+        double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+        if (CORR) { d0 = a.dwa_t[3 * c]; d1 = a.dwa_t[3 * c + 1]; d2 = a.dwa_t[3 * c + 2]; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = 4 * lane + i;
+          if (CORR) T.d[r][cl] = (d0 * f32_to_f64(F[0].v[i]) + d1 * f32_to_f64(F[1].v[i])) + d2 * f32_to_f64(F[2].v[i]);
+          else T.f[2][r][cl] = (cw.x * F[0].v[i] + cw.y * F[1].v[i]) + cw.z * F[2].v[i];
+          T.f[0][r][cl] = (g0 * Gt[0].v[i] + g1 * Gt[1].v[i] + g2 * Gt[2].v[i]) * cw.w;
+        }
+      }
+      {
+        const float h0 = G.kin_w32[3 * c], h1 = G.kin_w32[3 * c + 1], h2 = G.kin_w32[3 * c + 2];
+        const F4 a0 = ld4(a.a_e + E[0] + k), a1 = ld4(a.a_e + E[1] + k), a2 = ld4(a.a_e + E[2] + k);
+        const F4 w = ld4(a.w_stage + o + k), iz = ld4(G.inv_dz2_32 + k);
+        const float wm = k > 0 ? a.w_stage[o + k - 1] : 0.0f, wp = k + 4 <= N ? a.w_stage[o + k + 4] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float hadv = h0 * a0.v[i] + h1 * a1.v[i] + h2 * a2.v[i];
+          const float wu = i ? w.v[i ? i - 1 : 0] : wm, wd = i < 3 ? w.v[i < 3 ? i + 1 : 3] : wp;
+          T.f[1][4 * lane + i][cl] = -hadv - w.v[i] * (wu - wd) * iz.v[i];
+        }
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < LPE * CB; i += nthr) {
+      const int r = i / CB, cl = i % CB, kk = k0 + r;
+      const int64_t c = c0 + cl;
+      if (c >= nc || kk >= N) continue;
+      const int64_t j = (int64_t)kk * nc + c;
+      if (CORR) a.dr64[j] = T.d[r][cl];
+      else a.dr32[j] = T.f[2][r][cl];
+      a.dt32[j] = T.f[0][r][cl];
+      if (kk >= 1) {
+        float Aw = T.f[1][r][cl];
+        if (CORR) Aw = 0.5f * (a.Aw0[j] + Aw);
+        else a.Aw0[j] = Aw;
+        a.aw32[j] = dtau32 * Aw;
+      }
+    }
+    __syncthreads();
+  }
+}
 
 MxGeo make_mx_geo(const icon_grid* grid, const StateDev& s) {
   const GridDev& g = grid->g;
