@@ -948,7 +948,7 @@ struct MxLeanArgs {
   unsigned* status;
   double dtau, inv_nsub;
   int hdamp;                               // half levels h < hdamp are Rayleigh-damped
-  // corrector with divergence damping (fused into its gather): the undamped vn^{n+1}, the
+  // the ensemble's corrector with divergence damping (fused into its gather): the undamped vn^{n+1}, the
   // cell Laplacian of its divergence, the stage shadows for the fluxes, c4 Abar^2, the
   // damped vn^{n+1} (stored by each edge's lower-id cell, which also accumulates the
   // step-mean mass flux)
@@ -2396,7 +2396,7 @@ int ensemble_prepare(EnsembleDev& E, icon_state* const* members, int n, const do
     if (all_lean) {
       for (int stage = 0; stage < 2; ++stage) M.la[stage] = lean_args(s, stage == 1, dtau, nsub);
       if (M.damp) {
-        // as the per-state lean step: undamped vn^{n+1} in Avn0_32, damping fused into the gather
+        // undamped vn^{n+1} in Avn0_32 as in the per-state step; its edge update fused into the gather
         M.ea[1].vn_out = s.Avn0_32;
         M.dd.vn = s.Avn0_32;
         MxLeanArgs& la = M.la[1];
