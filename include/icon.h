@@ -295,7 +295,8 @@ int icon_global_mass_noalloc(const icon_grid* grid, const double* dev_rho, const
 /* Copy a field (icon_field) to host memory as FP64, [entity][level] unpadded;
  * count must equal the field's element count. Synchronous. Pinned (page-locked) host
  * memory is written directly by the packing kernel over the CPU-GPU link; other host
- * memory goes through a device staging buffer and one copy. */
+ * memory, a buffer that is page-locked only in part among it, goes through a device
+ * staging buffer and one copy. */
 int icon_state_copy_field(const icon_state* state, int field_id, double* host_dst, size_t count);
 
 /* Overwrite a prognostic field (ICON_F_VN .. ICON_F_EXNER) from FP64 host memory

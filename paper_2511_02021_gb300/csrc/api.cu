@@ -5,6 +5,8 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <cuda.h>
+#include "host_range.h"
 #include "icon_internal.h"
 
 namespace icon {
@@ -102,6 +104,36 @@ void DeviceArena::release() {
     else cudaFree(p);
   }
   blocks.clear();
+}
+
+// One contiguous copy between host and device memory. The driver refuses a host buffer that is
+// page-locked only in part, or in two registrations; such a one is copied in pieces through
+// pageable memory. Waits there; elsewhere the copy is as cudaMemcpyAsync's.
+cudaError_t copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t st) {
+  cudaError_t e = cudaMemcpyAsync(dst, src, bytes, kind, st);
+  if (e != cudaErrorInvalidValue) return e;
+  cudaGetLastError();
+  cudaPointerAttributes attr;                // device memory in place of host memory stays refused
+  if (cudaPointerGetAttributes(&attr, kind == cudaMemcpyHostToDevice ? src : dst) != cudaSuccess ||
+      attr.type == cudaMemoryTypeDevice) {
+    cudaGetLastError();
+    return e;
+  }
+  constexpr size_t kPiece = (size_t)1 << 20;
+  void* piece = malloc(kPiece);
+  if (!piece) return cudaErrorMemoryAllocation;
+  e = cudaSuccess;
+  for (size_t o = 0; o < bytes && e == cudaSuccess; o += kPiece) {
+    const size_t m = bytes - o < kPiece ? bytes - o : kPiece;
+    char* d = static_cast<char*>(dst) + o;
+    const char* s = static_cast<const char*>(src) + o;
+    if (kind == cudaMemcpyHostToDevice) memcpy(piece, s, m);
+    e = kind == cudaMemcpyHostToDevice ? cudaMemcpyAsync(d, piece, m, kind, st) : cudaMemcpyAsync(piece, s, m, kind, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && kind == cudaMemcpyDeviceToHost) memcpy(d, piece, m);
+  }
+  free(piece);
+  return e;
 }
 
 namespace {
@@ -420,21 +452,46 @@ bool field_ref(const icon_state* st, int id, void** ptr, int* is_f32, int64_t* n
   }
 }
 
-// the device address of n values of pinned (page-locked, mapped) host memory, or NULL for any
-// other pointer, for values that are not aligned, and where the last one is not in the same
-// mapping (a buffer registered in part); the queries allocate nothing
-double* mapped_host_ptr(const double* p, size_t n) {
-  auto device_ptr = [](const double* q) -> double* {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, q) != cudaSuccess) {
+// the page-locked range at a host address. The runtime says whether it is page-locked (and binds
+// the device's context to this thread), the driver where that allocation or registration begins
+// and ends; its entry point comes from the runtime, so nothing links against the driver
+HostRange pinned_range(uintptr_t p) {
+  using Attributes = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Attributes attributes = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) !=
+            cudaSuccess || found != cudaDriverEntryPointSuccess) {
       cudaGetLastError();
-      return nullptr;
+      f = nullptr;
     }
-    return attr.type == cudaMemoryTypeHost ? static_cast<double*>(attr.devicePointer) : nullptr;
-  };
-  if (n == 0 || reinterpret_cast<uintptr_t>(p) % alignof(double) != 0) return nullptr;
-  double* d = device_ptr(p);
-  return d && device_ptr(p + n - 1) == d + (n - 1) ? d : nullptr;
+    return reinterpret_cast<Attributes>(f);
+  }();
+  HostRange r;
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, reinterpret_cast<const void*>(p)) != cudaSuccess) {
+    cudaGetLastError();
+    return r;
+  }
+  if (attr.type != cudaMemoryTypeHost || !attr.devicePointer || !attributes) return r;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[] = {&start, &size};
+  if (attributes(2, what, out, (CUdeviceptr)p) != CUDA_SUCCESS) return r;
+  r.dev = reinterpret_cast<uintptr_t>(attr.devicePointer);
+  r.start = (uintptr_t)start;
+  r.size = size;
+  return r;
+}
+
+// the device address of n values of pinned (page-locked, mapped) host memory, or NULL for any
+// other pointer, for values that are not aligned, and where some of them are not page-locked (a
+// buffer registered in part); the queries allocate nothing
+double* mapped_host_ptr(const double* p, size_t n) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+  if (n == 0 || a % alignof(double) != 0) return nullptr;
+  return reinterpret_cast<double*>(mapped_address(a, n * sizeof(double), pinned_range));
 }
 
 // host-order [n][nlev] <-> the device rows of a field: FP64 or FP32 rows of ld
@@ -782,7 +839,7 @@ int icon_state_copy_field(const icon_state* st, int field_id, double* host_dst, 
   if (!stage) { set_error("icon_state_copy_field: out of device memory"); return ICON_ENOMEM; }
   cudaError_t e = move_field(ptr, stage, n, nlev, ld, f32 != 0, lm != 0, true, stream);
   if (e == cudaSuccess && !hd)
-    e = cudaMemcpyAsync(host_dst, stage, sizeof(double) * n * nlev, cudaMemcpyDeviceToHost, stream);
+    e = copy_host(host_dst, stage, sizeof(double) * n * nlev, cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   tmp.release();
   if (e != cudaSuccess) return cuda_fail(e, "icon_state_copy_field");
@@ -814,7 +871,7 @@ int icon_state_set_field(icon_state* st, int field_id, const double* host_src, s
   double* stage = hs ? hs : tmp.get_n<double>((size_t)n * nlev);
   if (!stage) { set_error("icon_state_set_field: out of device memory"); return ICON_ENOMEM; }
   cudaError_t e = cudaSuccess;
-  if (!hs) e = cudaMemcpyAsync(stage, host_src, sizeof(double) * n * nlev, cudaMemcpyHostToDevice, stream);
+  if (!hs) e = copy_host(stage, host_src, sizeof(double) * n * nlev, cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = move_field(ptr, stage, n, nlev, ld, f32 != 0, lm != 0, false, stream);
   if (e == cudaSuccess && lm) {
     mixed_refresh_shadows(st, stream);
@@ -964,10 +1021,10 @@ static int tracer_copy(icon_state* st, int t, double* host, size_t count, bool t
   tmp.al = st->arena.al;
   if (double* stage = hp ? hp : tmp.get_n<double>(count)) {
     cudaError_t e = cudaSuccess;
-    if (!to_host && !hp) e = cudaMemcpyAsync(stage, host, sizeof(double) * count, cudaMemcpyHostToDevice, stream);
+    if (!to_host && !hp) e = copy_host(stage, host, sizeof(double) * count, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = move_field(dev, stage, nc, N, ld, false, false, to_host, stream);
     if (e == cudaSuccess && to_host && !hp)
-      e = cudaMemcpyAsync(host, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, stream);
+      e = copy_host(host, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     tmp.release();
     if (e != cudaSuccess) return cuda_fail(e, fn);

@@ -628,7 +628,7 @@ int icon_domain_copy_field(icon_domain* D, int field_id, double* host_dst, size_
                                                                   src[field_id], stage);
     }
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(host_dst, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = copy_host(host_dst, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     tmp.release();
     if (e != cudaSuccess) return cuda_fail(e, "icon_domain_copy_field");

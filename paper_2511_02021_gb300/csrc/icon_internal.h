@@ -58,6 +58,8 @@ struct Allocator {
 };
 Allocator current_allocator();
 cudaStream_t current_stream();
+// a copy between host and device memory that takes any host buffer (api.cu)
+cudaError_t copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t st);
 
 // A set of device buffers released together with the allocator that made them.
 struct DeviceArena {
