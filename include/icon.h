@@ -324,7 +324,7 @@ int icon_dycore_step_profile(icon_state* state, double dt, int nsubsteps, double
  * NaN included; binary32 subnormals to a signed zero), and the Newton-Raphson FP64
  * reciprocal of the column solves is
  * compared with the IEEE division on n random operands (within 1 ulp for 1/x,
- * 2 ulps for a * (1/x)), the FP64 square root of the diffusion with the IEEE one (1 ulp). *failures receives the number of mismatches (0 expected).
+ * 2 ulps for a * (1/x)). *failures receives the number of mismatches (0 expected).
  * Allocates 4 bytes with cudaMalloc (not the registered allocator). Waits. */
 int icon_selftest(long long n, unsigned* failures);
 

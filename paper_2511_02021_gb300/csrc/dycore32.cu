@@ -1785,8 +1785,8 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
   prof_end(stream);
 }
 
-// ---------------------------------------------------------------- self-test of the integer-pipe conversions,
-// the Newton-Raphson reciprocal and the square root
+// ---------------------------------------------------------------- self-test of the integer-pipe conversions
+// and of the Newton-Raphson reciprocal
 namespace {
 __device__ inline uint64_t st_mix(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -1845,12 +1845,6 @@ __global__ void k_selftest_conv(int64_t n, unsigned* fails) {
   const double q2 = av / xv, y2 = av * recip64(xv);
   const long long dq2 = __double_as_longlong(q2) - __double_as_longlong(y2);
   if (dq2 > 2 || dq2 < -2) atomicAdd(fails, 1u);
-  // square root: within one ulp of the IEEE root, of positive x with exponents in [-500, 500]
-  const uint64_t ex5 = 523u + (r4 >> 50) % 1001u;
-  const double sx = __longlong_as_double((long long)((r4 & 0x000fffffffffffffull) | (ex5 << 52)));
-  const long long dq3 = __double_as_longlong(sqrt(sx)) - __double_as_longlong(sqrt64(sx));
-  if (dq3 > 1 || dq3 < -1) atomicAdd(fails, 1u);
-  if (i == 0 && sqrt64(0.0) != 0.0) atomicAdd(fails, 1u);
 }
 }  // namespace
 

@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(256, 3) k_diff_edge(Geo64 G, double* __restric
                       fma(d12z, t12[2], fma(d12y, t12[1], d12x * t12[0]));
     const double DS = fma(d12z, n12[2], fma(d12y, n12[1], fma(d12x, n12[0],
                       fma(d34z, t34[2], fma(d34y, t34[1], d34x * t34[0])))));
-    const double D = sqrt64(fma(DS, DS, DT * DT));
+    const double D = sqrt(fma(DS, DS, DT * DT));
     const double lap = (divc[c2 + k] - divc[c1 + k]) * ide - (zeta[v2 + k] - zeta[v1 + k]) * ile;
     double vnew = fma(dtk * D, lap, vn[e * ld + k]);
     if (bd.D1) {

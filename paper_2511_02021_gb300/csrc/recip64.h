@@ -1,4 +1,4 @@
-// FP64 reciprocal (Newton-Raphson refinement of a binary32 seed) and square root.
+// FP64 reciprocal by Newton-Raphson refinement of a binary32 seed.
 //
 // An IEEE FP64 division issues about eight FP64-pipe operations on this GPU, whose
 // FP64 pipe retires one warp instruction per SM every 16 cycles; the column solves
@@ -31,21 +31,6 @@ __device__ __forceinline__ double recip64(double x) {
   const double e = fma(-x, y0, 1.0);
   const double t = fma(e, e, e);
   return fma(y0, t, y0);
-}
-
-// FP64 square root of x >= 0 from an approximate reciprocal square root y0 (relative error
-// below 2^-20, full exponent range, not on the FP64 pipe): with g = x y0 and e = 1 - x y0^2,
-//   sqrt(x) = g (1 - e)^(-1/2) = g (1 + e/2 + 3 e^2/8 + ...), truncated after e^2,
-// five FP64 operations and a relative error of order e^3 < 2^-56, so within one ulp. Zero
-// and subnormal x (whose root is below 2^-511) give 0.
-__device__ __forceinline__ double sqrt64(double x) {
-  double y0;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  const double g = x * y0;
-  const double e = fma(-g, y0, 1.0);
-  const double t = e * fma(0.375, e, 0.5);
-  const double r = fma(g, t, g);
-  return (__double2hiint(x) & 0x7ff00000) ? r : 0.0;
 }
 
 }  // namespace icon
