@@ -278,17 +278,21 @@ int alloc_state(icon_state* st, int precision, bool topo) {
     s.wflx = A.get_n<double>(C);
     s.colconst = A.get_n<double>(8 * (size_t)ld);
     double** col[] = {&s.col_lo, &s.col_di, &s.col_up, &s.col_rh, &s.col_rx,
-                      &s.col_tx, &s.col_px, &s.col_gm, &s.col_ri, &s.col_mm, &s.col_ws, &s.col_gc};
+                      &s.col_gm, &s.col_ri, &s.col_mm, &s.col_ws, &s.col_gc};
     for (double** p : col) *p = A.get_n<double>(C);
     if (!topo) s.col_d0 = A.get_n<double>(C);
     s.vn = A.get_n<double>(E); s.vn_s = A.get_n<double>(E);
     s.Avn0 = A.get_n<double>(E); s.Aw0 = A.get_n<double>(C);
     s.zeta = A.get_n<double>(V); s.w_v = A.get_n<double>(V);
-    s.vt = A.get_n<double>(E); s.Ke = A.get_n<double>(E); s.Kc = A.get_n<double>(C);
+    s.vt = A.get_n<double>(E > C ? E : C); s.Ke = A.get_n<double>(E > C ? E : C); s.Kc = A.get_n<double>(C);
     s.a_e = A.get_n<double>(E); s.F = A.get_n<double>(E); s.G = A.get_n<double>(E);
     s.kin_w_h = A.get_n<double>(3 * (size_t)nc); s.div_wa_h = A.get_n<double>(3 * (size_t)nc);
     s.adv_w = A.get_n<double>(3 * (size_t)nc);
     s.edge_c = A.get_n<double>(4 * (size_t)ne); s.lap_w = A.get_n<double>(4 * (size_t)nc);
+    // the edge tendency reads vt last and the cells' kinetic energy Ke: the column of the same
+    // stage keeps its explicit parts of Theta and Exner there, from its rows to its update (col_d0,
+    // which lasts from one stage to the next, is a field of its own)
+    s.col_tx = s.Ke; s.col_px = s.vt;
     // diffusion scratch reuses substep scratch (they never overlap in time)
     s.thflx = s.Ke; s.divc = s.Kc; s.uvx = s.w_v;
     s.uvy = A.get_n<double>(V); s.uvz = A.get_n<double>(V);
