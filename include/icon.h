@@ -461,7 +461,7 @@ void icon_domain_free(icon_domain* domain);
  * picks them on the first step (timing every candidate on the state's data, in the order
  * of the step; cached per grid size, level count and GPU, and in the file named by the
  * environment variable ICON_TUNE_CACHE if set). The lean column (24): its launch form,
- * lanes 2 and block one of 9 (chosen by the grid's size, the default), 6 or 8 (blocks of
+ * lanes 2 and block one of 9 (chosen by the grid's cells and levels, the default), 6 or 8 (blocks of
  * four or eight warps per 32 columns), 10 or 12 (one column per thread, its loads one or
  * two levels ahead), the same in both stages. set_tiling forces a tile (lanes 0 restores
  * automatic choice; ICON_EINVAL for any other value outside these sets); results do not

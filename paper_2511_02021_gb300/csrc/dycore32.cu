@@ -41,6 +41,7 @@
 #include <string>
 #include <type_traits>
 #include "icon_internal.h"
+#include "lean_rule.h"
 #include "fastconv.h"
 #include "recip64.h"
 
@@ -1539,7 +1540,7 @@ void launch_mx_column(const MxGeo& G, const MxColArgs& a, bool topo, cudaStream_
 // ---------------------------------------------------------------- autotuner
 // Candidate tiles over (entity, level): 32 lanes per entity (one entity per warp), 16
 // (two per warp) or 8 (four per warp), blocks of 64, 128, 256 or 512 threads: twelve per
-// stencil kind. (The lean column's form follows a rule on the grid's size, lean_form, and its
+// stencil kind. (The lean column's form follows a rule on cells and levels, lean_rule.h, and its
 // gather has one shape.) Each kind is timed on the state's own data (three launches
 // per candidate after one untimed, CUDA events) and the fastest kept, in the order of the
 // step, so that every trial reads inputs its predecessors formed. Choices are cached per
@@ -1636,7 +1637,7 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   // a trial that met a non-finite value would have flagged the state; the step that
   // follows checks it again
   cudaMemsetAsync(s.status, 0, sizeof(unsigned), stream);
-  // the lean column's form follows the grid's size and its gather has one shape
+  // the lean column's form follows cells and levels and its gather has one shape
   if (lean && !st->tile_forced[K_MX_LEAN]) st->tile[K_MX_LEAN] = kLeanDefault;
   if (lean && !st->tile_forced[K_MX_COLUMN_PREP]) st->tile[K_MX_COLUMN_PREP] = TileChoice{8, 256};
   st->tuned = true;

@@ -23,6 +23,7 @@
 //     81,920 x 90              320 / 403   250 / 295    273 / 397
 //     327,680 x 90            1058 / 1159  954 / 1074  1047 / 1479
 //     81,920 x 90, terrain     449 / 546   390 / 394    490 / 639
+// Which one a state runs: lean_rule.h.
 //
 // Both forms, at every shape, give the same bits: which of two products is rounded before the
 // multiply-add that takes the other is written out, not left to how the compiler contracts a
@@ -408,12 +409,6 @@ __global__ void __launch_bounds__(kLeanThreads, kLeanBlocks) k_mx_lean_column(Mx
   }
   if (!ok && act) atomicOr(a.status, 1u);
 #undef LMV
-}
-
-constexpr int kLeanPitch = 33;             // shared row pitch: conflict-free by columns and by levels
-inline size_t lean_tile_bytes(int N, bool topo) {
-  return (size_t)N * kLeanPitch * (sizeof(double) + 3 * sizeof(float)) +
-         (topo ? (size_t)(N + 1) * kLeanPitch * sizeof(float) : 0);
 }
 
 // one block of W warps per 32 columns; 660 (over terrain 792) bytes of shared memory per level.
@@ -841,8 +836,6 @@ __global__ void __launch_bounds__(32 * W, MINB) k_mx_lean_tile(MxGeo G, MxLeanAr
 #undef LMV
 }
 
-// launch forms of the lean column (the tile of kind K_MX_LEAN: lanes 2, block one of these)
-enum { LEAN_TILE4 = 6, LEAN_TILE8 = 8, LEAN_RULE = 9, LEAN_COLUMN1 = 10, LEAN_COLUMN2 = 12 };
 const TileChoice kLeanDefault = {2, LEAN_RULE};
 
 bool lean_shape_ok(const TileChoice& t) {
@@ -850,18 +843,16 @@ bool lean_shape_ok(const TileChoice& t) {
                           t.block == LEAN_COLUMN1 || t.block == LEAN_COLUMN2);
 }
 
-// The form by size: tiles of 32 columns per SM. Up to three, a tile has an SM nearly to itself
-// and eight warps shorten its parallel parts; up to eight, four warps a tile (20,480 columns,
-// 4.2 tiles per SM: 53 / 72 us against 82 / 97 one column per thread); beyond, enough warps of
-// columns fill the SMs (81,920 columns, 16.8 tiles per SM, 90 levels: 250 / 295 us against
-// 273 / 397 by tiles).
+// the forced form, or the one lean_rule.h gives for the current device
 int lean_form(const MxGeo& G, const TileChoice& t, bool topo) {
   if (t.block != LEAN_RULE) return t.block;
-  const int64_t tiles = (G.nc + 31) / 32;
-  constexpr int64_t kSMs = 152;
-  if (tiles <= 3 * kSMs) return LEAN_TILE8;
-  if (tiles <= 8 * kSMs) return LEAN_TILE4;
-  return topo ? LEAN_COLUMN1 : LEAN_COLUMN2;
+  int dev = 0, sms = 152, shared = 233472, reserved = 1024;      // a GB300's, should a query fail
+  if (cudaGetDevice(&dev) == cudaSuccess) {
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&shared, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  }
+  return lean_form_for(G.nc, G.N, topo, sms, (size_t)shared, (size_t)reserved);
 }
 
 template <bool CORR, bool TOPO, int W, int MINB>
