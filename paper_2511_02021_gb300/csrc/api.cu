@@ -1005,6 +1005,23 @@ int icon_state_tracers(const icon_state* st, int* out) {
   return ICON_OK;
 }
 
+// Whether a tracer crosses to or from host memory row by row (cudaMemcpy2D, no kernel and no buffer)
+// or as one packed run: by the time per call measured on a GB300, rows / packed, us.
+//   pinned: the run is moved by the packing kernel itself. Rows of whole 128-byte lines go at the
+//     link's rate either way (set R2B4/96 85 / 86), others a row at a time (R2B4/60 594 / 60, read back
+//     112 / 64); very short ones save the launch (R2B2/8 9 / 11; R2B5/2 37 / 18).
+//   pageable: the run takes a device buffer and a second pass, about 8 us whatever the size. Reading back
+//     up to 1,280 rows costs less (R2B2/20 16 / 19, R2B3/20 29 / 22); rows of 128 levels and more
+//     are long enough up to 5,120 of them (R2B3/256 66 / 78; R2B4/128 165 / 137), those of 224 at any
+//     number (R2B5/256 908 / 965); setting, where short rows cost more, up to 320 rows (R2B0/90
+//     13 / 18, R2B1/90 21 / 24, R2B2/90 48 / 28) or 1,280 of whole lines (R2B2/128 16 / 31).
+static bool tracer_by_rows(int64_t nc, int N, bool pinned, bool to_host) {
+  if (pinned) return N % 16 == 0 || (N <= 8 && nc <= 5120) || (to_host && nc <= 80);
+  if (N <= 4 && nc <= 20480) return true;
+  if (to_host) return nc <= 1280 || N >= 224 || (N >= 128 && nc <= 5120);
+  return nc <= 320 || (nc <= 1280 && (N % 16 == 0 || N <= 8));
+}
+
 static int tracer_copy(icon_state* st, int t, double* host, size_t count, bool to_host) {
   const char* fn = to_host ? "icon_state_copy_tracer" : "icon_state_set_tracer";
   if (!st || !host) { set_error("%s: NULL argument", fn); return ICON_EINVAL; }
@@ -1017,28 +1034,35 @@ static int tracer_copy(icon_state* st, int t, double* host, size_t count, bool t
   }
   double* dev = st->s.q + (size_t)t * nc * ld;
   cudaStream_t stream = current_stream();
-  // through a packed device buffer and one contiguous transfer (or the pinned buffer itself): a
-  // strided copy of 480-byte rows to pageable memory took 20 ms per tracer at R2B5 / 60 levels
-  // (39 MB). Row by row only where the buffer does not fit
   double* hp = mapped_host_ptr(host, count);
+  auto by_rows = [&] {
+    cudaError_t e = to_host ? cudaMemcpy2DAsync(host, sizeof(double) * N, dev, sizeof(double) * ld, sizeof(double) * N,
+                                                nc, cudaMemcpyDeviceToHost, stream)
+                            : cudaMemcpy2DAsync(dev, sizeof(double) * ld, host, sizeof(double) * N, sizeof(double) * N,
+                                                nc, cudaMemcpyHostToDevice, stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(stream) : e;
+  };
+  if (tracer_by_rows(nc, N, hp != nullptr, to_host)) {
+    const cudaError_t e = by_rows();
+    if (e == cudaSuccess) return ICON_OK;
+    if (e != cudaErrorInvalidValue) return cuda_fail(e, fn);     // else: host memory registered in part
+    cudaGetLastError();
+  }
+  // through a packed device buffer and one contiguous transfer, or the pinned buffer itself; row by
+  // row where there is no room for the buffer
   DeviceArena tmp;
   tmp.al = st->arena.al;
+  cudaError_t e = cudaSuccess;
   if (double* stage = hp ? hp : tmp.get_n<double>(count)) {
-    cudaError_t e = cudaSuccess;
     if (!to_host && !hp) e = copy_host(stage, host, sizeof(double) * count, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = move_field(dev, stage, nc, N, ld, false, false, to_host, stream);
     if (e == cudaSuccess && to_host && !hp)
       e = copy_host(host, stage, sizeof(double) * count, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     tmp.release();
-    if (e != cudaSuccess) return cuda_fail(e, fn);
-    return ICON_OK;
+  } else {
+    e = by_rows();
   }
-  cudaError_t e = to_host ? cudaMemcpy2DAsync(host, sizeof(double) * N, dev, sizeof(double) * ld, sizeof(double) * N,
-                                              nc, cudaMemcpyDeviceToHost, stream)
-                          : cudaMemcpy2DAsync(dev, sizeof(double) * ld, host, sizeof(double) * N, sizeof(double) * N,
-                                              nc, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, fn);
   return ICON_OK;
 }
