@@ -519,29 +519,35 @@ __global__ void k_pack(const T* __restrict__ src, double* __restrict__ host, int
 // two orders cross in shared memory, so both sides are coalesced. Writing R2B6 / 90 levels (vn
 // and four level-major fields, 1.3 GB) to pinned memory took 33 ms with one word per thread in
 // device order, a row's stride apart in a staging buffer that was then copied; 6.9 ms now, a
-// field's 236 MB at 188 GB/s, the link's rate.
-constexpr int kPackThreads = 256;
+// field's 236 MB at 188 GB/s, the link's rate. A block takes kc levels: all of them or, on grids
+// with fewer blocks of 32 entities than SMs, 32 (blockIdx.y: the chunk; R2B1/256, ten blocks: 24.7 us
+// a copy to pageable memory, 21.4 in chunks; R2B3/90, 160 blocks, to pinned memory: 30.8 and 34.2).
+constexpr int kPackThreads = 256, kPackChunk = 32, kPackWholeBlocks = 152;
 __global__ void __launch_bounds__(kPackThreads) k_pack_lm(const double* __restrict__ src, double* __restrict__ host,
-                                                          int64_t n, int nlev) {
-  extern __shared__ double pack_tile[];                      // [nlev][33]
+                                                          int64_t n, int nlev, int kc) {
+  extern __shared__ double pack_tile[];                      // [kc][33]
   const int64_t c0 = (int64_t)blockIdx.x * 32;
   const int m = (int)(n - c0 < 32 ? n - c0 : 32), cl = threadIdx.x & 31;
+  const int k0 = blockIdx.y * kc, nk = nlev - k0 < kc ? nlev - k0 : kc;
   if (cl < m)
-    for (int k = threadIdx.x >> 5; k < nlev; k += kPackThreads / 32) pack_tile[k * 33 + cl] = src[(int64_t)k * n + c0 + cl];
+    for (int k = threadIdx.x >> 5; k < nk; k += kPackThreads / 32)
+      pack_tile[k * 33 + cl] = src[(int64_t)(k0 + k) * n + c0 + cl];
   __syncthreads();
-  double* out = host + c0 * nlev;
-  for (int t = threadIdx.x; t < m * nlev; t += kPackThreads) out[t] = pack_tile[(t % nlev) * 33 + t / nlev];
+  double* out = host + c0 * nlev + k0;
+  for (int t = threadIdx.x; t < m * nk; t += kPackThreads) out[t / nk * nlev + t % nk] = pack_tile[(t % nk) * 33 + t / nk];
 }
 __global__ void __launch_bounds__(kPackThreads) k_unpack_lm(const double* __restrict__ host, double* __restrict__ dst,
-                                                            int64_t n, int nlev) {
+                                                            int64_t n, int nlev, int kc) {
   extern __shared__ double pack_tile[];
   const int64_t c0 = (int64_t)blockIdx.x * 32;
   const int m = (int)(n - c0 < 32 ? n - c0 : 32), cl = threadIdx.x & 31;
-  const double* in = host + c0 * nlev;
-  for (int t = threadIdx.x; t < m * nlev; t += kPackThreads) pack_tile[(t % nlev) * 33 + t / nlev] = in[t];
+  const int k0 = blockIdx.y * kc, nk = nlev - k0 < kc ? nlev - k0 : kc;
+  const double* in = host + c0 * nlev + k0;
+  for (int t = threadIdx.x; t < m * nk; t += kPackThreads) pack_tile[(t % nk) * 33 + t / nk] = in[t / nk * nlev + t % nk];
   __syncthreads();
   if (cl < m)
-    for (int k = threadIdx.x >> 5; k < nlev; k += kPackThreads / 32) dst[(int64_t)k * n + c0 + cl] = pack_tile[k * 33 + cl];
+    for (int k = threadIdx.x >> 5; k < nk; k += kPackThreads / 32)
+      dst[(int64_t)(k0 + k) * n + c0 + cl] = pack_tile[k * 33 + cl];
 }
 
 // a field's device buffer to (pack) or from host order; `host` is device-addressable
@@ -549,13 +555,17 @@ cudaError_t move_field(void* field, double* host, int64_t n, int nlev, int ld, b
                        cudaStream_t stream) {
   const unsigned nb = blocks_for(n * nlev, 256);
   if (lm) {
-    const size_t sm = sizeof(double) * 33 * nlev;            // at most 67,848 B (257 half levels)
-    cudaError_t e = cudaFuncSetAttribute(k_pack_lm, cudaFuncAttributeMaxDynamicSharedMemorySize, 33 * 257 * 8);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_unpack_lm, cudaFuncAttributeMaxDynamicSharedMemorySize, 33 * 257 * 8);
-    if (e != cudaSuccess) return e;
-    if (pack) k_pack_lm<<<blocks_for(n, 32), kPackThreads, sm, stream>>>(static_cast<double*>(field), host, n, nlev);
-    else k_unpack_lm<<<blocks_for(n, 32), kPackThreads, sm, stream>>>(host, static_cast<double*>(field), n, nlev);
+    const unsigned blocks = blocks_for(n, 32);
+    const int kc = blocks < kPackWholeBlocks && nlev > kPackChunk ? kPackChunk : nlev;
+    const dim3 grid(blocks, blocks_for(nlev, kc));
+    const size_t sm = sizeof(double) * 33 * kc;              // at most 67,848 B (257 half levels)
+    if (sm > (48 << 10)) {                                   // what a launch has to ask for
+      const cudaError_t e = cudaFuncSetAttribute(pack ? (const void*)k_pack_lm : (const void*)k_unpack_lm,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 33 * 257 * 8);
+      if (e != cudaSuccess) return e;
+    }
+    if (pack) k_pack_lm<<<grid, kPackThreads, sm, stream>>>(static_cast<double*>(field), host, n, nlev, kc);
+    else k_unpack_lm<<<grid, kPackThreads, sm, stream>>>(host, static_cast<double*>(field), n, nlev, kc);
   } else if (f32) {
     if (pack) k_pack<<<nb, 256, 0, stream>>>(static_cast<const float*>(field), host, n, nlev, ld);
     else k_unpack<<<nb, 256, 0, stream>>>(host, static_cast<float*>(field), n, nlev, ld);
