@@ -312,7 +312,9 @@ int icon_state_step_kernels(icon_state* state, double dt, int nsubsteps, int* ou
 /* Run one step eagerly (not from the graph) with a CUDA event pair around every
  * kernel launch and add each launch's duration (ms) to ms_per_kind[kind] and 1 to
  * launches_per_kind[kind] (host arrays of ICON_KIND_COUNT entries, accumulated,
- * not cleared). The state advances exactly as with icon_dycore_step. Waits. */
+ * not cleared). A launch that vertices and edges share on a small grid (FP64 up to 5,120
+ * cells, mixed up to 20,480 unless a tile of either is forced) counts as the vertices'.
+ * The state advances exactly as with icon_dycore_step. Waits. */
 int icon_dycore_step_profile(icon_state* state, double dt, int nsubsteps, double* ms_per_kind,
                              int* launches_per_kind);
 
@@ -456,16 +458,18 @@ void icon_domain_free(icon_domain* domain);
 /* ---------------------------------------------------------------- ensemble */
 
 /* Tile of a kernel kind (the kind numbers of icon_kernel_kind_name) of a mixed-precision
- * state. Stencil kinds (10, 11, 12, 13, 15, 16): lanes per entity (32 = one entity per
- * warp, 16 = two, 8 = four) and threads per block (64, 128, 256 or 512); the autotuner
- * picks them on the first step (timing every candidate on the state's data, in the order
- * of the step; cached per grid size, level count and GPU, and in the file named by the
- * environment variable ICON_TUNE_CACHE if set). The lean column (24): its launch form,
- * lanes 2 and block one of 9 (chosen by the grid's cells and levels, the default), 6 or 8 (blocks of
- * four or eight warps per 32 columns), 10 or 12 (one column per thread, its loads one or
- * two levels ahead), the same in both stages. set_tiling forces a tile (lanes 0 restores
- * automatic choice; ICON_EINVAL for any other value outside these sets); results do not
- * depend on the tile. */
+ * state. Stencil kinds (10, 11, 12, 13, 16, and 15, the gather of the stored-factor column;
+ * the lean column's gather, 25, has one shape, whatever is set for 15): lanes per entity
+ * (32 = one entity per warp, 16 = two, 8 = four) and threads per block (64, 128, 256 or
+ * 512). The autotuner picks them on the first step (timing every candidate on the state's
+ * data, in the order of the step; cached per grid size, level count and GPU, and in the
+ * file named by the environment variable ICON_TUNE_CACHE if set). On grids up to 20,480
+ * cells kinds 10 and 11 run in one launch of (8, 128), and apart once a tile of either is
+ * forced. The lean column (24): its launch form, lanes 2 and block one of 9 (chosen by the
+ * grid's cells and levels, the default), 6 or 8 (blocks of four or eight warps per 32
+ * columns), 10 or 12 (one column per thread, its loads one or two levels ahead), the same
+ * in both stages. set_tiling forces a tile (lanes 0 restores automatic choice; ICON_EINVAL
+ * for any other value outside these sets); results do not depend on the tile. */
 int icon_state_tiling(const icon_state* state, int kind, int* lanes, int* block);
 int icon_state_set_tiling(icon_state* state, int kind, int lanes, int block);
 

@@ -1490,7 +1490,6 @@ void launch_kind(int kind, const TileChoice& t, const MxGeo& G, StateDev& s, con
     case K_MX_EDGE_TEND:
       with_lanes(t.lanes, [&](auto L) {
         constexpr int LPE = decltype(L)::value;
-        const int B = t.block < 256 ? t.block : 256;       // 85 registers for three such blocks per SM
         if (s.topo.on) k_mx_edge_tend<LPE, true><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
         else k_mx_edge_tend<LPE, false><<<item_blocks(G.ne, LPE, B), B, 0, st>>>(G, ea);
       });
@@ -1589,6 +1588,14 @@ void save_tune_entry(const std::string& key, const TileChoice& t) {
 
 }  // namespace
 
+// Up to R2B4 the vertices and the edge diagnostics share a launch: there a launch runs about as long
+// as starting it takes (R2B4/60: 1.275 -> 1.239 ms per step). A forced tile of either kind keeps
+// them apart, each in its own.
+static bool merges_vertex_edge(const icon_state* st) {
+  constexpr int64_t kMergeMaxCells = 20480;
+  return st->grid->g.nc <= kMergeMaxCells && !st->tile_forced[K_MX_VERTEX] && !st->tile_forced[K_MX_EDGE];
+}
+
 bool lean_column_shape_ok(int lanes, int form) { return lean_shape_ok(TileChoice{lanes, form}); }
 
 void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
@@ -1598,12 +1605,16 @@ void autotune_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream) {
   // the predictor's arguments: every tuned kernel then writes only scratch or S* buffers
   const MxEdgeArgs ea = edge_args(s, false, dtau, nsub);
   const MxColArgs ca = col_args(s, false, dtau, nsub);
-  const bool lean = s.ln_B != nullptr;
+  const bool lean = s.ln_B != nullptr, merged = merges_vertex_edge(st);
   std::lock_guard<std::mutex> lk(g_tune_mu);
   load_tune_file();
   for (int kind : kTunedKinds) {
     if (st->tile[kind].lanes != 0 && st->tile_forced[kind]) continue;
     if (kind == K_MX_COLUMN_PREP && !s.fac64) continue;
+    if (merged && (kind == K_MX_VERTEX || kind == K_MX_EDGE)) {
+      st->tile[kind] = TileChoice{8, 128};                       // the merged launch's
+      continue;
+    }
     const std::string key = tune_key(kind, G);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
@@ -1668,7 +1679,8 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
   // what the branch saves (64 states of R2B4/60 and R2B5/60 stepped one after another: 270 ->
   // 285 ms), over terrain and for the FP64 step the branch measured slower or equal: it is
   // recorded for flat mixed states of at least kBranchMinCells cells (R2B6) only.
-  constexpr int64_t kBranchMinCells = 327680, kMergeMaxCells = 20480;
+  constexpr int64_t kBranchMinCells = 327680;
+  const bool merged = merges_vertex_edge(st);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(stream, &cs);
   const bool overlap = lean && !s.topo.on && nc >= kBranchMinCells && st->side_stream &&
@@ -1694,10 +1706,8 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
       ead.skip_flux = damp ? 1 : 0;
       ead.upwind_theta = st->upwind_theta ? 1 : 0;
       for (int kind : {K_MX_VERTEX, K_MX_EDGE, K_MX_CELL_KE, K_MX_EDGE_TEND}) {
-        // up to R2B4 (20,480 cells) the vertices and the edge diagnostics share a launch: there a
-        // launch runs about as long as starting it takes (R2B4/60: 1.275 -> 1.239 ms per step)
-        if (nc <= kMergeMaxCells && kind == K_MX_EDGE) continue;
-        if (nc <= kMergeMaxCells && kind == K_MX_VERTEX) {
+        if (merged && kind == K_MX_EDGE) continue;
+        if (merged && kind == K_MX_VERTEX) {
           const unsigned nbv = blocks_for(G.nv, 16);
           prof_begin(stream, kind);
           k_mx_vertex_edge<<<nbv + blocks_for(G.ne, 16), 128, 0, stream>>>(G, ead.vn, ead.w, s.zeta32, s.wv32, s.vt32, nbv);

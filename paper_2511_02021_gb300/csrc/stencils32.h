@@ -286,8 +286,9 @@ __device__ __forceinline__ void mx_edge_tend_quads(const MxGeo& G, const MxEdgeA
   }
 }
 
+// 64 registers, so 1,024 threads per SM in blocks of any size the tile may have
 template <int LPE, bool TOPO>
-__global__ void __launch_bounds__(256, 4) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
+__global__ void __launch_bounds__(512, 2) k_mx_edge_tend(MxGeo G, MxEdgeArgs a) {
   QUAD_PROLOGUE(LPE, G.ne)
   mx_edge_tend_quads<LPE, TOPO>(G, a, item, lane);
 }
