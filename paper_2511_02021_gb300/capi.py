@@ -325,7 +325,7 @@ def icon_ensemble_phase_name(phase):
 # mixed-precision stencil kinds that take a tile
 KIND_MX_VERTEX, KIND_MX_EDGE, KIND_MX_CELL_KE, KIND_MX_EDGE_TEND, KIND_MX_COLUMN_PREP, KIND_MX_DIFF_VERTEX = \
     10, 11, 12, 13, 15, 16
-# the lean mixed column: its tile is a launch form (2, form); (2, 9) follows the grid's size
+# the lean mixed column: its tile is a launch form (2, form); (2, 9) follows the grid's cells and levels
 KIND_MX_LEAN = 24
 LEAN_SHAPES = ((2, 9), (2, 10), (2, 8), (2, 12), (2, 6))
 

@@ -961,13 +961,13 @@ struct MxLeanArgs {
   // terrain-following levels (TOPO instances): the column's per-cell tables, level-major
   // [k][Nc] (upper interpolation weight, 1/dz, 1/dzh, reference Exner), the stage's
   // contravariant correction wcc at half levels ([Nc][ld]); for the gather w - wcc and 1/dzh
-  // ([Nc][ld]) and the layer thickness at edges ([Ne][ld])
+  // ([Nc][ld])
   const double *t_wu_lm, *t_idz_lm, *t_idzh_lm, *t_exref_lm;
-  const float *t_wcc, *t_wcon, *t_inv_dzh, *t_dz_e;
+  const float *t_wcc, *t_wcon, *t_inv_dzh;
 };
 
-// per-warp shadow transpose: CH levels of 32 columns (16 in the per-state kernel, 8 in the
-// persistent ensemble, whose blocks hold four warps' tiles)
+// per-warp shadow transpose: CH levels of 32 columns (eight, per state and in the persistent
+// ensemble)
 template <int CH>
 struct LeanTile {
   float t[4][CH][33];                      // rho, theta_v, pi - pi_ref, w of 32 columns
@@ -1109,7 +1109,7 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
   // half levels k and k+1); the level above (k-1) is loaded one step ahead for the
   // half-level interpolants
   bool ok = true;
-  double x_next = 0.0, wn_next = 0.0;                // half level k+1: undamped, damped
+  double x_next = 0.0;                               // half level k+1, undamped
   float wnf_next = 0.f;
   // half level k+1 quantities carried upward
   float ri_next = 0.f, M_next = 0.f, xv_next = 0.f;  // at k+1 (explicit vertical velocity of S^n)
@@ -1195,7 +1195,6 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     T.t[3][k - k0][lane] = wnf;
     if (k == k0) lean_flush(G, a, T, c0, k0, lane);
     x_next = x;
-    wn_next = wn;
     wnf_next = wnf;
     ri_next = ri_k;
     M_next = M_k;
@@ -1204,7 +1203,6 @@ __device__ inline void mx_lean_column_item(const MxGeo& G, const MxLeanArgs& a, 
     thv_k = thv_u;
     ex_k = ex_u;
   }
-  (void)wn_next;
   if (act) {
     a.w32[cc * ld + N] = 0.0f;
     if (CORR) LMV(a.w, N) = 0.0;                   // the ground (w^n there is 0 already)
@@ -1422,7 +1420,7 @@ MxLeanArgs lean_args(StateDev& s, bool corr, double dtau, int nsub) {
   la.dd_upwind = 0;
   const TopoDev& T = s.topo;
   la.t_wu_lm = T.wu_lm; la.t_idz_lm = T.idz_lm; la.t_idzh_lm = T.idzh_lm; la.t_exref_lm = T.exref_lm;
-  la.t_wcc = T.wcc32; la.t_wcon = T.wcon32; la.t_inv_dzh = T.inv_dzh_c32; la.t_dz_e = T.dz_e32;
+  la.t_wcc = T.wcc32; la.t_wcon = T.wcon32; la.t_inv_dzh = T.inv_dzh_c32;
   return la;
 }
 
@@ -1674,11 +1672,12 @@ void enqueue_step_mixed(icon_state* st, double dt, int nsub, cudaStream_t stream
   // and write vt32 and Kc32, which neither this stage's gather nor its column reads. While a
   // step on flat levels is recorded into its graph they go on a second branch beside the
   // column, whose last wave of blocks leaves part of the SMs idle; the branch is joined before
-  // the next stage's edge tendency. Eager (profiled) steps keep one stream. Measured: R2B6/90
-  // 29.5 -> 28.7 ms per step, R2B8/90 439.7 -> 438.5 ms; on coarser grids the joins cost about
-  // what the branch saves (64 states of R2B4/60 and R2B5/60 stepped one after another: 270 ->
-  // 285 ms), over terrain and for the FP64 step the branch measured slower or equal: it is
-  // recorded for flat mixed states of at least kBranchMinCells cells (R2B6) only.
+  // the next stage's edge tendency. Eager (profiled) steps keep one stream. Measured, one branch ->
+  // two: R2B6/90 21.98 -> 21.39 ms per step, R2B6/47 12.84 -> 12.40, R2B7/90 83.2 -> 82.4, R2B8/90
+  // 324.7 -> 324.0; R2B5/90 5.97 -> 5.88, R2B4/60 1.24 -> 1.29 ms, where the joins cost what the
+  // branch saves or more. Over terrain and for the FP64 step it measured slower or equal with the
+  // kernels of its time. It is recorded for flat mixed states of at least kBranchMinCells cells
+  // (R2B6) only.
   constexpr int64_t kBranchMinCells = 327680;
   const bool merged = merges_vertex_edge(st);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -2401,7 +2400,8 @@ int ensemble_prepare(EnsembleDev& E, icon_state* const* members, int n, const do
     if (all_lean) {
       for (int stage = 0; stage < 2; ++stage) M.la[stage] = lean_args(s, stage == 1, dtau, nsub);
       if (M.damp) {
-        // undamped vn^{n+1} in Avn0_32 as in the per-state step; its edge update fused into the gather
+        // undamped vn^{n+1} in Avn0_32, which the gather's edge update reads (the per-state step
+        // damps vn32 in place, in a kernel of its own)
         M.ea[1].vn_out = s.Avn0_32;
         M.dd.vn = s.Avn0_32;
         MxLeanArgs& la = M.la[1];

@@ -197,8 +197,8 @@ struct EdgeArgs {
   double* vn_out;                          // vn* or vn^{n+1} (may alias vn_base)
   double* Avn0;                            // stored (predictor) or read (corrector)
   double *F, *G, *a_e, *mflx;
-  double dtau, inv_nsub;
-  double hinv_nsub;                        // inv_nsub / 2 (set on the host)
+  double dtau;
+  double hinv_nsub;                        // 1 / (2 nsub), set on the host
   double hdtau;                            // dtau / 2 (set on the host)
   int corrector;
   int skip_flux;                           // fluxes formed after divergence damping instead
@@ -929,9 +929,9 @@ Geo64 make_geo(const icon_grid* grid, const double* cc) {
 }
 
 // Merged launches on small grids, whose kernels run 2 to 4 us, about what starting one takes: the
-// column's three parts up to R2B2 (1,280 cells; 90 launches per step of R2B2/20 398 us, merged 356;
-// on R2B3/90 the parts fill the SMs better apart, 2334 against 2887 us), vertices with edges up
-// to R2B3.
+// column's three parts up to R2B2 (1,280 cells; R2B2/20 398 us a step with 90 launches, 356 merged,
+// R2B2/60 791 and 724; on R2B3 the parts fill the SMs better apart, R2B3/30 765 us against 900,
+// R2B3/90 2286 against 2887), vertices with edges up to R2B3 (R2B3/30 785 us apart, 765 merged).
 constexpr int64_t kMergeColumnCells = 1280, kMergeStencilCells = 5120;
 
 template <bool TOPO, bool CORR>
@@ -1025,7 +1025,7 @@ void fp64_step_stage(icon_state* st, double dt, int nsub, bool corr, cudaStream_
   ea.vn_out = corr ? s.vn : s.vn_s;
   ea.Avn0 = s.Avn0;
   ea.F = s.F; ea.G = s.G; ea.a_e = s.a_e; ea.mflx = s.mflx;
-  ea.dtau = dtau; ea.inv_nsub = 1.0 / nsub; ea.corrector = corr;
+  ea.dtau = dtau; ea.corrector = corr;
   ea.hinv_nsub = 0.5 / nsub;
   ea.hdtau = 0.5 * dtau;
   const bool damp = corr && st->divdamp4 > 0.0;

@@ -33,7 +33,11 @@
 __device__ __forceinline__ float lean_g(double ex, float rhof, float thvf) {
   return __fmul_rn(kRcvF, __fdividef(f64_to_f32(ex), __fmul_rn(rhof, thvf)));
 }
-// a b - c d with one product rounded before the subtraction: the second (FIRST) or the first
+// a b - c d with one product rounded before the subtraction: the second (FIRST) or the first. Results
+// are defined by the loop these forms replaced, whose body was unrolled by two and in which the
+// compiler fused one product at even steps of a sweep and the other at odd ones: the upward sweep
+// below takes its levels in the same pairs (ODD), and so does the last row of the corrector, whose
+// difference of Exner increments was fused when the row fell on the pair's first step (even N).
 template <bool FIRST>
 __device__ __forceinline__ float fma_diff(float a, float b, float c, float d) {
   return FIRST ? __fmaf_rn(a, b, -__fmul_rn(c, d)) : __fmaf_rn(-c, d, __fmul_rn(a, b));
@@ -189,6 +193,7 @@ __global__ void __launch_bounds__(kLeanThreads, kLeanBlocks) k_mx_lean_column(Mx
           } else {
             B = v.B;
           }
+          // an even N's last row as the unrolled loop rounded it (see fma_diff)
           const float dd = (CORR && j == N && (N & 1) == 0) ? __fmaf_rn(-g, dthe, dpe2) : __fsub_rn(dpe2, dpe1);
           const float inc = __fmaf_rn(-aa, dd, v.aw);
           const float lo = __fmul_rn(__fmul_rn(-aa, gam2), M2);
@@ -567,6 +572,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_mx_lean_tile(MxGeo G, MxLeanAr
             } else {
               B = v.B;
             }
+            // an even N's last row as the unrolled loop rounded it (see fma_diff)
             const float dd = (CORR && j == N && (N & 1) == 0) ? __fmaf_rn(-g, dthe, dpe2) : __fsub_rn(dpe2, dpe1);
             const float inc = __fmaf_rn(-aa, dd, v.aw);
             const int i = h * PT + lane;
